@@ -355,7 +355,7 @@ size_t layout_problem(ProbHost& h) {
     h.lay.tile_frames = o;
     o = align_up(o + sizeof(int) * std::max(h.tile_frames.size(), (size_t)p.J * per_frame));
     h.lay.pos_part = o;
-    o = align_up(o + 5 * sizeof(double) * (size_t)p.J * ((p.N + 7) / 8));
+    o = align_up(o + 5 * sizeof(double) * (size_t)p.J * pos_bands(p.N));
     // CG: gradient, previous gradient and direction of object and probe
     h.lay.cg_obj = o;
     o = align_up(o + 3 * sizeof(float2) * (size_t)p.Ho * p.Wo);
@@ -1648,10 +1648,7 @@ ptx_status ptx_position_shifts(ptx_handle* h, int32_t p, float filter_ratio, flo
     ptx_status st = check_device(h);
     if (st != PTX_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int bands = (ph.p.N + 7) / 8;
-    double* part = (double*)(h->scratch + ph.lay.pos_part);
-    k_pos_sums<<<dim3(bands, ph.p.J), 256, 0, s>>>(ph.args, part);
-    k_pos_solve<<<1, 1024, 0, s>>>(part, ph.p.J, bands, filter_ratio, shifts);
+    launch_position_shifts(ph.args, (double*)(h->scratch + ph.lay.pos_part), filter_ratio, shifts, s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ptx_position_shifts launch");
     return PTX_OK;

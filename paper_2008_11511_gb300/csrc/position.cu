@@ -12,74 +12,142 @@
 namespace ptx {
 
 namespace {
-
-__device__ __forceinline__ float2 obj_at(const ProbArgs& a, int y, int x) { return a.obj[(size_t)y * a.Wo + x]; }
-
-// dO/dy, dO/dx at (y, x) of the object
-__device__ __forceinline__ void obj_grad(const ProbArgs& a, int y, int x, float2& gy, float2& gx) {
-    const int y0 = y > 0 ? y - 1 : y, y1 = y < a.Ho - 1 ? y + 1 : y;
-    const int x0 = x > 0 ? x - 1 : x, x1 = x < a.Wo - 1 ? x + 1 : x;
-    const float sy = 1.0f / (float)(y1 - y0), sx = 1.0f / (float)(x1 - x0);
-    gy = cscale(csub(obj_at(a, y1, x), obj_at(a, y0, x)), sy);
-    gx = cscale(csub(obj_at(a, y, x1), obj_at(a, y, x0)), sx);
-}
-
+constexpr int kPosSum = 8;             // rows summed in FP32 by a thread
+constexpr int kPosRows = 2 * kPosSum;  // rows each thread walks down
+// pairs of adjacent columns, and rows of such pairs a block of 256 threads holds
+__host__ __device__ inline int pos_groups(int N) { return 256 / (N / 2); }
 }  // namespace
 
-// grid (rows / 8 bands, J): block sums the five products of its 8 rows of frame j
-// over all modes and writes them to part[(j * bands + band) * 5 + q] (FP64).
-__global__ void __launch_bounds__(256) k_pos_sums(ProbArgs a, double* part) {
-    __shared__ double red[5][8];
+int pos_bands(int N) {
+    const int rows = pos_groups(N) * kPosRows;
+    return (N + rows - 1) / rows;
+}
+
+// grid (J, bands): a block sums the five products of its rows of frame j over
+// all modes and writes them to part[(j * bands + band) * 5 + q] (FP64).
+//
+// Bound: the exit waves are read once from HBM, everything else comes from L2
+// and L1.  A thread owns two adjacent columns and walks down kPosRows rows with
+// the object rows y - 1, y, y + 1 of its columns in registers, so each object
+// pixel is loaded for its own row only (and twice for the neighbours'
+// columns), the probe and the exit wave by 16-byte loads, and no index is
+// divided inside the loop.  With |G|^2 = |P|^2 |dO|^2 and Re(conj(P dO) chi) =
+// Re(conj(dO) w), w = sum_k conj(P_k) Psi_k - |P|^2 O, a mode costs one complex
+// product and |P|^2 instead of three products and five sums.
+// A thread's sums over kPosSum rows stay in FP32, the block's are FP64.
+// Sixteen rows per thread re-read 2 halo rows in 18 (8 rows: 2 in 10), and four
+// blocks per SM leave the registers for four rows of loads in flight.
+// 1000 frames of 256^2, all three launches: 1108 -> 203 us (start: every product
+// from global memory, FP64 shuffles in every warp, one block for all the solves);
+// 8 rows per thread 213, 32 rows 177 but with longer FP32 sums than before.
+template <bool kOneMode>
+__global__ void __launch_bounds__(256, kOneMode ? 4 : 3) k_pos_sums(ProbArgs a, double* part) {
+    __shared__ float part_s[2][5][256];
     const int N = a.N, K = a.K;
-    const int band = blockIdx.x, j = blockIdx.y;
-    const int2 p = a.pos[j];
-    float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // yy, yx, xx, y.chi, x.chi
-    for (int e = threadIdx.x; e < 8 * N; e += blockDim.x) {
-        const int y = band * 8 + e / N, x = e % N;
-        if (y >= N) break;
-        float2 gy, gx;
-        obj_grad(a, p.x + y, p.y + x, gy, gx);
-        const float2 o = obj_at(a, p.x + y, p.y + x);
-        for (int k = 0; k < K; ++k) {
-            const size_t pix = ((size_t)k * N + y) * N + x;
-            const float2 pr = __ldg(a.probe + pix);
-            const float2 chi = csub(a.psi[(size_t)j * K * N * N + pix], cmul(pr, o));
-            const float2 Gy = cmul(pr, gy), Gx = cmul(pr, gx);
-            s[0] += cnorm(Gy);
-            s[1] += Gy.x * Gx.x + Gy.y * Gx.y;
-            s[2] += cnorm(Gx);
-            s[3] += Gy.x * chi.x + Gy.y * chi.y;
-            s[4] += Gx.x * chi.x + Gx.y * chi.y;
+    const int j = blockIdx.x, band = blockIdx.y;
+    const int pairs = N / 2, groups = pos_groups(N);
+    const int grp = threadIdx.x / pairs, x = 2 * (threadIdx.x - grp * pairs);
+    const int y_first = (band * groups + grp) * kPosRows;
+    float s[2][5] = {};  // per half of the rows: yy, yx, xx, y.chi, x.chi
+    if (grp < groups && y_first < N) {
+        const int2 p = a.pos[j];
+        const int c = p.y + x;                                       // object columns c, c + 1
+        const int cl = c > 0 ? c - 1 : c, cr = c + 2 < a.Wo ? c + 2 : c + 1;  // their outer neighbours
+        const float sx0 = c > 0 ? 0.5f : 1.0f, sx1 = c + 2 < a.Wo ? 0.5f : 1.0f;
+        const int r = p.x + y_first;
+        const float2* row = a.obj + (size_t)r * a.Wo;
+        const float2* up = r > 0 ? row - a.Wo : row;
+        float2 m0 = up[c], m1 = up[c + 1];                            // row y - 1 (clamped)
+        float2 ol = row[cl], o0 = row[c], o1 = row[c + 1], oh = row[cr];  // row y
+        const size_t f0 = (size_t)y_first * N + x;
+        const float2* psi = a.psi + (size_t)j * K * N * N + f0;
+        const float2* pr = a.probe + f0;
+        const int rows = min(kPosRows, N - y_first);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll 4
+          for (int i = h * kPosSum; i < min(rows, (h + 1) * kPosSum); ++i) {
+            const bool last = r + i + 1 >= a.Ho, first = r + i == 0;
+            const float2* down = last ? row : row + a.Wo;
+            const float2 nl = down[cl], n0 = down[c], n1 = down[c + 1], nh = down[cr];
+            const float sy = (last || first) ? 1.0f : 0.5f;
+            float p0 = 0.f, p1 = 0.f;
+            float2 w0 = make_float2(0.f, 0.f), w1 = w0;
+#pragma unroll 1
+            for (int k = 0; k < (kOneMode ? 1 : K); ++k) {
+                const size_t o = (size_t)k * N * N + (size_t)i * N;
+                const float4 q = __ldg(reinterpret_cast<const float4*>(pr + o));
+                const float4 v = __ldcs(reinterpret_cast<const float4*>(psi + o));
+                p0 = fmaf(q.x, q.x, fmaf(q.y, q.y, p0));
+                p1 = fmaf(q.z, q.z, fmaf(q.w, q.w, p1));
+                w0 = cadd(w0, cconjmul(make_float2(q.x, q.y), make_float2(v.x, v.y)));
+                w1 = cadd(w1, cconjmul(make_float2(q.z, q.w), make_float2(v.z, v.w)));
+            }
+            const float2 gy0 = cscale(csub(n0, m0), sy), gx0 = cscale(csub(o1, ol), sx0);
+            const float2 gy1 = cscale(csub(n1, m1), sy), gx1 = cscale(csub(oh, o0), sx1);
+            w0 = make_float2(fmaf(-p0, o0.x, w0.x), fmaf(-p0, o0.y, w0.y));
+            w1 = make_float2(fmaf(-p1, o1.x, w1.x), fmaf(-p1, o1.y, w1.y));
+            s[h][0] = fmaf(p0, cnorm(gy0), fmaf(p1, cnorm(gy1), s[h][0]));
+            s[h][1] = fmaf(p0, fmaf(gy0.x, gx0.x, gy0.y * gx0.y), fmaf(p1, fmaf(gy1.x, gx1.x, gy1.y * gx1.y), s[h][1]));
+            s[h][2] = fmaf(p0, cnorm(gx0), fmaf(p1, cnorm(gx1), s[h][2]));
+            s[h][3] += fmaf(gy0.x, w0.x, fmaf(gy0.y, w0.y, fmaf(gy1.x, w1.x, gy1.y * w1.y)));
+            s[h][4] += fmaf(gx0.x, w0.x, fmaf(gx0.y, w0.y, fmaf(gx1.x, w1.x, gx1.y * w1.y)));
+            m0 = o0; m1 = o1;
+            ol = nl; o0 = n0; o1 = n1; oh = nh;
+            row = down;
+          }
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // FP64 across the threads: warp q < 5 adds product q of all of them (one
+    // FP64 addition per value; shuffling FP64 sums in every warp took 100 us
+    // more at 1000 x 256^2, FP64 throughput being a few lanes per clock)
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        double v = (double)s[q];
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) part_s[h][q][threadIdx.x] = s[h][q];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 5) {
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v += (double)part_s[i >> 3][warp][lane + 32 * (i & 7)];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[q][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-        part[((size_t)j * gridDim.x + band) * 5 + threadIdx.x] = v;
+        if (lane == 0) part[((size_t)j * gridDim.y + band) * 5 + warp] = v;
     }
 }
 
-// One block: per-frame sums in band order, the mean gradient norm, the solves.
-__global__ void __launch_bounds__(1024) k_pos_solve(const double* part, int J, int bands, float filter_ratio,
+// One warp per frame adds the frame's bands (in a fixed order) into the first
+// band's five entries.  Apart from the solve so that the frames' bands are read
+// by the whole GPU.
+__global__ void __launch_bounds__(256) k_pos_frame(double* part, int J, int bands) {
+    const int j = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (j >= J) return;
+    double* f = part + (size_t)j * bands * 5;
+    double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int b = lane; b < bands; b += 32)
+        for (int q = 0; q < 5; ++q) m[q] += f[b * 5 + q];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[q] += __shfl_down_sync(0xffffffffu, m[q], o);
+    }
+    __syncwarp();
+    if (lane == 0)
+        for (int q = 0; q < 5; ++q) f[q] = m[q];
+}
+
+// Block b solves frames 256 b .. 256 b + 255.  Every block adds all the frames'
+// norms itself, in the same order (the mean decides which frames are filtered):
+// J doubles from L2 cost less than a launch in between, and the FP64 divisions of
+// the solves, which one block alone would queue for 20 us at J = 1000, spread out.
+__global__ void __launch_bounds__(256) k_pos_solve(const double* part, int J, int bands, float filter_ratio,
                                                     float* shifts) {
     __shared__ double red[32];
     double nsum = 0.0;
     for (int j = threadIdx.x; j < J; j += blockDim.x) {
-        double yy = 0.0, xx = 0.0;
-        for (int b = 0; b < bands; ++b) {
-            yy += part[((size_t)j * bands + b) * 5 + 0];
-            xx += part[((size_t)j * bands + b) * 5 + 2];
-        }
-        nsum += yy + xx;
+        const double* m = part + (size_t)j * bands * 5;
+        nsum += m[0] + m[2];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nsum += __shfl_down_sync(0xffffffffu, nsum, o);
@@ -88,10 +156,9 @@ __global__ void __launch_bounds__(1024) k_pos_solve(const double* part, int J, i
     double total = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) total += red[w];
     const double mean = total / (double)J;
-    for (int j = threadIdx.x; j < J; j += blockDim.x) {
-        double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int b = 0; b < bands; ++b)
-            for (int q = 0; q < 5; ++q) m[q] += part[((size_t)j * bands + b) * 5 + q];
+    const int j = blockIdx.x * 256 + threadIdx.x;
+    if (j < J) {
+        const double* m = part + (size_t)j * bands * 5;
         const double norm = m[0] + m[2];
         const double det = m[0] * m[2] - m[1] * m[1];
         float dy = 0.f, dx = 0.f;
@@ -102,6 +169,16 @@ __global__ void __launch_bounds__(1024) k_pos_solve(const double* part, int J, i
         shifts[2 * j] = dy;
         shifts[2 * j + 1] = dx;
     }
+}
+
+void launch_position_shifts(const ProbArgs& a, double* part, float filter_ratio, float* shifts, cudaStream_t s) {
+    const int bands = pos_bands(a.N);
+    if (a.K == 1)
+        k_pos_sums<true><<<dim3(a.J, bands), 256, 0, s>>>(a, part);
+    else
+        k_pos_sums<false><<<dim3(a.J, bands), 256, 0, s>>>(a, part);
+    if (bands > 1) k_pos_frame<<<(a.J + 7) / 8, 256, 0, s>>>(part, a.J, bands);
+    k_pos_solve<<<(a.J + 255) / 256, 256, 0, s>>>(part, a.J, bands, filter_ratio, shifts);
 }
 
 }  // namespace ptx

@@ -1,0 +1,47 @@
+"""Kernels at the sizes where they can go wrong: edges of tiles, remainders of
+chunks, the smallest and largest of their range, each against 64-bit results."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2008_11511_gb300 import build as b
+    b.build()
+
+
+def crandn(rng, *shape):
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+
+def dev(x):
+    return torch.tensor(np.ascontiguousarray(x), device="cuda")
+
+
+@pytest.mark.parametrize("N,K,J", [(8, 1, 3), (12, 2, 2), (80, 1, 5), (224, 3, 3), (256, 1, 40), (400, 2, 2), (512, 1, 2)])
+def test_position_shifts_at_edges(N, K, J):
+    """Frames on the object's corners and edges (one-sided differences), sizes
+    whose rows do not fill the last band, several modes."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + K)
+    Ho, Wo = N + 5, N + 2
+    obj = (1 + 0.3 * crandn(rng, Ho, Wo)).astype(np.complex64)
+    probe = crandn(rng, K, N, N)
+    pos = np.stack([rng.integers(0, Ho - N + 1, J), rng.integers(0, Wo - N + 1, J)], 1).astype(np.int32)
+    pos[0], pos[1] = (0, 0), (Ho - N, Wo - N)
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)
+    psi = (phi * (1 + 0.1 * crandn(rng, *phi.shape))).astype(np.complex64)
+    pb = Ptycho(dev(obj), dev(probe), torch.zeros((J, N, N), device="cuda"), pos, psi=dev(psi))
+    got = pb.position_shifts(0.0).cpu().numpy()
+    ref = oracle.position_shifts(obj, probe, psi, pos, 0.0)
+    # the sums are of N^2 K terms of random sign and size |G| |chi|, |chi| ~ 0.1 |G| here: each term is good to
+    # 2^-21, so the shift to about 2^-21 * 0.1 * sqrt(2); 1e-5 leaves room for the condition of the 2 x 2 system
+    assert np.abs(got - ref).max() < 1e-5
+    pb.close()
