@@ -25,6 +25,21 @@ def dev(x):
     return torch.tensor(np.ascontiguousarray(x), device="cuda")
 
 
+# (N, frames): one frame, frames that fit one block, several chunks with a remainder
+@pytest.mark.parametrize("N,frames", [(32, 1), (64, 3), (64, 700), (80, 5), (128, 513), (256, 300), (400, 53), (512, 35)])
+@pytest.mark.parametrize("direction", [-1, 1])
+def test_fft2_chunks_and_remainders(N, frames, direction):
+    from paper_2008_11511_gb300 import fft2
+    g = torch.Generator(device="cuda").manual_seed(N + frames)
+    x = torch.view_as_complex(torch.randn(frames, N, N, 2, generator=g, device="cuda"))
+    f = torch.fft.fft2 if direction < 0 else torch.fft.ifft2
+    ref = f(x.to(torch.complex128), norm="ortho")
+    fft2(x, direction)
+    per_frame = (x - ref).abs().square().sum((1, 2)).sqrt() / ref.abs().square().sum((1, 2)).sqrt()
+    # 2 log2 N butterfly levels, each within a few units of 2^-24
+    assert float(per_frame.max()) < 2 * np.log2(N) * 2.0 ** -24
+
+
 @pytest.mark.parametrize("N,K,J", [(8, 1, 3), (12, 2, 2), (80, 1, 5), (224, 3, 3), (256, 1, 40), (400, 2, 2), (512, 1, 2)])
 def test_position_shifts_at_edges(N, K, J):
     """Frames on the object's corners and edges (one-sided differences), sizes
