@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_fft_rows_r
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < S::I1; ++i) {
-        const int w = threadIdx.x + i * kThreads;
+        const int w = row_item<N, M>(i);
         if (w < L * M) {
             const int line = w / M, n1 = w - line * M;
             const float2* src = base + line * N + n1;
@@ -52,11 +52,11 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_fft_rows_r
             for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, DIR>(tw, k2, n1));
         }
     }
-    __syncthreads();
+    row_sync<N>();
     pdl_wait();
 #pragma unroll
     for (int i = 0; i < S::I2; ++i) {
-        const int w = threadIdx.x + i * kThreads;
+        const int w = row_item<N, R>(i);
         if (w < L * R) {
             const int line = w / R, k2 = w - line * R;
             const float2* src = buf + line * P + k2 * (M + 1);
