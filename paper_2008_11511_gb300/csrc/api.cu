@@ -362,7 +362,7 @@ size_t layout_problem(ProbHost& h) {
     h.lay.cg_probe = o;
     o = align_up(o + 3 * sizeof(float2) * (size_t)p.K * p.N * p.N);
     h.lay.ls_part = o;
-    o = align_up(o + 2 * sizeof(double) * (size_t)p.J * (p.N / ls_cols(h.ks, p.K)));
+    o = align_up(o + 2 * sizeof(double) * (size_t)p.J * (p.N / ls_cols(h.ks)));
     h.lay.cg = o;
     o = align_up(o + (8 + 3 * (size_t)kCgBlocks) * sizeof(double));  // scalars, then the dot-product partials
     h.lay.mbits = o;
@@ -561,8 +561,10 @@ ptx_status compute_layout(std::vector<ProbHost>& probs, size_t* spec_off, size_t
         h.lay.pos_part += o;
         h.lay.end += o;
         o += sz;
-        size_t s = (size_t)h.B * kDefaultLanes * h.p.K * h.p.N * h.p.N * sizeof(float2);
-        if (s > spec) spec = s;
+        // at least the three waves per mode of one frame of the line search (more
+        // than the lanes' slices hold when there is a single frame)
+        const size_t frame = (size_t)h.p.K * h.p.N * h.p.N * sizeof(float2);
+        spec = std::max(spec, std::max((size_t)h.B * kDefaultLanes, (size_t)3) * frame);
         frames += (size_t)h.p.J;
     }
     *ctl_off = o;
@@ -1323,8 +1325,8 @@ ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj,
     a.dir_obj = d_obj;
     a.dir_probe = d_probe;
     // work stack per frame: the waves A, B (and C with both parts of the
-    // direction) of one mode for the register kernels, 3 K waves otherwise
-    const int waves = (ph.p.K == 1 && ph.ks->reg_lines > 0) ? ((d_obj && d_probe) ? 3 : 2) : 3 * ph.p.K;
+    // direction) of every mode for the register kernels, always three otherwise
+    const int waves = (ph.ks->reg_lines > 0 ? ls_waves(d_obj, d_probe) : 3) * ph.p.K;
     const size_t frame_w = (size_t)waves * ph.p.N * ph.p.N * sizeof(float2);
     size_t B = h->spec_bytes / frame_w;
     if (B < 1) B = 1;
@@ -1337,7 +1339,7 @@ ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj,
         ph.ks->col_ls(a, j0, nb, pdl, s);
     }
     // partial pairs per frame: one per column block of the line-search column pass
-    k_ls_reduce<<<1, 1024, 0, s>>>(a.ls_part, (size_t)ph.p.J * (ph.p.N / ls_cols(ph.ks, ph.p.K)), out);
+    k_ls_reduce<<<1, 1024, 0, s>>>(a.ls_part, (size_t)ph.p.J * (ph.p.N / ls_cols(ph.ks)), out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "line-search launch");
     return PTX_OK;

@@ -347,14 +347,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_r(ProbArgs a, int j0, i
 }
 
 // ---------------------------------------------------------------------------
-// ML line search, one probe mode (the same arithmetic as k_row_fwd_ls /
-// k_col_ls, with the register-resident transforms).  For a direction (dO, dP)
-// the far field along the line is A + a B + a^2 C with A = FT(P O),
+// ML line search (the same arithmetic as k_row_fwd_ls / k_col_ls, which serve
+// the one-pass sizes, with the register-resident transforms).  For a direction
+// (dO, dP) the far field along the line is A + a B + a^2 C with A = FT(P O),
 // B = FT(dP O + P dO), C = FT(dP dO); C vanishes unless both parts of the
 // direction are given.
 //
-// Row pass: grid (N / L, frames in batch, waves), blockIdx.z = wave (0: A,
-// 1: B, 2: C); row transforms into spec[b][wave] (gridDim.z waves per frame).
+// Row pass: grid (N / L, frames in batch, waves x K), blockIdx.z = wave * K +
+// mode (waves 0: A, 1: B, 2: C); row transforms into spec[b][wave][mode].
 // ---------------------------------------------------------------------------
 template <int N>
 __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls_r(ProbArgs a, int j0) {
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
     load_twiddles<N>(tw);
     const int y0 = blockIdx.x * L;
     const int b = blockIdx.y;
-    const int wave = blockIdx.z;
+    const int wave = blockIdx.z / a.K, k = blockIdx.z - wave * a.K;
     const int2 p = a.pos[j0 + b];
     __syncthreads();
 #pragma unroll
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
         if (w < L * M) {
             const int line = w / M, n1 = w - line * M;
             const int y = y0 + line;
-            const size_t pi = (size_t)y * N + n1;
+            const size_t pi = ((size_t)k * N + y) * N + n1;
             const size_t oi = (size_t)(p.x + y) * a.Wo + p.y + n1;
             float2 v[R];
 #pragma unroll
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
 #pragma unroll
             for (int n1 = 0; n1 < M; ++n1) u[n1] = src[n1];
             Dft<M, -1>::run(u);
-            float2* dst = a.spec + (((size_t)b * gridDim.z + wave) * N + y0 + line) * N + k2;
+            float2* dst = a.spec + (((size_t)b * gridDim.z + blockIdx.z) * N + y0 + line) * N + k2;
             const uint64_t el = policy_evict_last();
 #pragma unroll
             for (int k1 = 0; k1 < M; ++k1) st_hint(dst + R * k1, u[k1], el);
@@ -423,69 +423,92 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
     }
 }
 
-// Blocks per SM of the line-search column pass: it holds A, the d2I partial
-// and one more wave per pixel in registers.
-template <int N>
+// Blocks per SM of the line-search column pass, from the values a thread holds
+// per pixel: A and B, the d2I partial with a third wave, the three sums over
+// modes with several modes.
+template <int N, bool kModes, bool kThree>
 __host__ __device__ constexpr int ls_min_blocks() {
-    return Plan<N>::M >= 20 ? 1 : 2;
+    const int regs = (4 + (kModes ? 3 : (kThree ? 1 : 0))) * RegShape<N>::CI2 * Plan<N>::M;
+    return regs <= 64 ? 3 : (regs <= 112 ? 2 : 1);
 }
 
-// Column pass: column transforms of the waves (A first, then C, then B, so
-// that the reduction runs on B while it is in registers) and the FP64 sums
+// Column pass: column transforms of the waves of every mode and the FP64 sums
 //   L'(0)  = sum (1 - I_o/I_c) dI,  L''(0) = sum [(1 - I_o/I_c) d2I + (I_o/I_c^2) dI^2]
-// with dI = 2 Re(conj(A) B), d2I = 2 |B|^2 + 4 Re(conj(A) C), over unmasked
-// pixels; one (L', L'') pair per block into ls_part[j][blockIdx.x].  The
+// with dI = 2 sum_k Re(conj(A) B), d2I = 2 sum_k (|B|^2 + 2 Re(conj(A) C)), over
+// unmasked pixels; one (L', L'') pair per block into ls_part[j][blockIdx.x].  The
 // per-pixel terms are single precision (I_o dI^2 / I_c^2 as I_o (dI / I_c)^2,
 // which stays finite at the I_c floor), summed with compensation per thread and
 // in FP64 across the block.  grid (N / C, frames in batch).
-template <int N>
-__global__ void __launch_bounds__(kThreads, ls_min_blocks<N>()) k_col_ls_r(ProbArgs a, int j0, int nwaves) {
+//
+// Bound: latency of the stack loads and of the two shared-memory round trips.
+// A and B go through their first factor together, each in a buffer of its own,
+// so that both waves' loads are in flight at once and a block meets two
+// barriers per mode; without a third wave the 64 values of a thread's pixels
+// leave room for three blocks per SM.
+template <int N, bool kModes, bool kThree>
+__global__ void __launch_bounds__(kThreads, (ls_min_blocks<N, kModes, kThree>())) k_col_ls_r(ProbArgs a, int j0) {
     using S = RegShape<N>;
     constexpr int R = S::R, M = S::M, C = S::C, P = S::P;
+    constexpr int kWaves = kThree ? 3 : 2;
     extern __shared__ __align__(16) float2 sm[];
     __shared__ double red_s[kThreads / 32];
     float2* tw = sm;
-    float2* buf = sm + N;
+    float2* buf0 = sm + N;
+    float2* buf1 = buf0 + C * P;
     pdl_launch_dependents();
     load_twiddles<N>(tw);
+    const int K = kModes ? a.K : 1;
     const int x0 = blockIdx.x * C;
     const int b = blockIdx.y;
     const int j = j0 + b;
     constexpr float invN2 = 1.0f / float(N * N);
-    float2 A[S::CI2][M];
-    float d2[S::CI2][M];
-    KahanF l1, l2;  // per-pixel terms in single precision (FP64 throughput is low), compensated sums
+    const float2* spec = a.spec + (size_t)b * K * kWaves * N * N + x0;
+    float2 A[S::CI2][M], B[S::CI2][M];
+    // sums over the modes; one mode needs d2 only, and only with a third wave
+    float ic_s[kModes ? S::CI2 : 1][kModes ? M : 1], di_s[kModes ? S::CI2 : 1][kModes ? M : 1];
+    float d2_s[kModes || kThree ? S::CI2 : 1][kModes || kThree ? M : 1];
+    if constexpr (kModes) {
+#pragma unroll
+        for (int i = 0; i < S::CI2; ++i)
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) ic_s[i][k1] = di_s[i][k1] = d2_s[i][k1] = 0.f;
+    }
+    // first factor of a wave's columns from registers into a buffer
+    auto load1 = [&](float2* v, const float2* w, int n1, int c) {
+#pragma unroll
+        for (int n2 = 0; n2 < R; ++n2) v[n2] = __ldcs(w + (size_t)(n1 + M * n2) * N + c);
+    };
+    auto pass1 = [&](float2* v, float2* buf, int n1, int c) {
+        Dft<R, -1>::run(v);
+        float2* o = buf + c * P + n1;
+        o[0] = v[0];
+#pragma unroll
+        for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, -1>(tw, k2, n1));
+    };
+    auto pass2 = [&](float2* u, const float2* buf, int k2, int c) {
+        const float2* src = buf + c * P + k2 * (M + 1);
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) u[n1] = src[n1];
+        Dft<M, -1>::run(u);
+    };
     __syncthreads();
     // launched as a programmatic dependent of the row pass that writes the work stack
     pdl_wait();
-    for (int s = 0; s < nwaves; ++s) {
-        const int wave = s == 0 ? 0 : (s == nwaves - 1 ? 1 : 2);
-        const float2* spec = a.spec + ((size_t)b * nwaves + wave) * N * N + x0;
+    for (int k = 0; k < K; ++k) {
+        const float2* wa = spec + (size_t)k * N * N;  // wave w of mode k: (w K + k) N^2
+        const float2* wb = wa + (size_t)K * N * N;
+        const float2* wc = wb + (size_t)K * N * N;
+        // A with C (kept for d2I), then B; without C, A and B together
 #pragma unroll
         for (int i = 0; i < S::CI1; ++i) {
             const int w = threadIdx.x + i * kThreads;
             if (w < C * M) {
                 const int n1 = w / C, c = w - n1 * C;
-                float2 v[R];
-#pragma unroll
-                for (int n2 = 0; n2 < R; ++n2) v[n2] = __ldcs(spec + (size_t)(n1 + M * n2) * N + c);
-                Dft<R, -1>::run(v);
-                float2* o = buf + c * P + n1;
-                o[0] = v[0];
-#pragma unroll
-                for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, -1>(tw, k2, n1));
-            }
-        }
-        __syncthreads();
-        float2 u[S::CI2][M];
-#pragma unroll
-        for (int i = 0; i < S::CI2; ++i) {
-            const int w = threadIdx.x + i * kThreads;
-            if (w < C * R) {
-                const int k2 = w / C, c = w - k2 * C;
-                const float2* src = buf + c * P + k2 * (M + 1);
-#pragma unroll
-                for (int n1 = 0; n1 < M; ++n1) u[i][n1] = src[n1];
+                float2 va[R], vb[R];
+                load1(va, wa, n1, c);
+                load1(vb, kThree ? wc : wb, n1, c);
+                pass1(va, buf0, n1, c);
+                pass1(vb, buf1, n1, c);
             }
         }
         __syncthreads();
@@ -494,38 +517,88 @@ __global__ void __launch_bounds__(kThreads, ls_min_blocks<N>()) k_col_ls_r(ProbA
             const int w = threadIdx.x + i * kThreads;
             if (w < C * R) {
                 const int k2 = w / C, c = w - k2 * C;
-                Dft<M, -1>::run(u[i]);
-                if (s == 0) {
+                pass2(A[i], buf0, k2, c);
+                pass2(B[i], buf1, k2, c);
+                if constexpr (kThree) {
 #pragma unroll
                     for (int k1 = 0; k1 < M; ++k1) {
-                        A[i][k1] = u[i][k1];
-                        d2[i][k1] = 0.f;
-                    }
-                } else if (wave == 2) {
-#pragma unroll
-                    for (int k1 = 0; k1 < M; ++k1)
-                        d2[i][k1] = 4.f * (A[i][k1].x * u[i][k1].x + A[i][k1].y * u[i][k1].y) * invN2;
-                } else {
-                    uint32_t mbits = 0u;
-                    if (a.mbits) mbits = a.mbits[blockIdx.x * kThreads + threadIdx.x] >> (i * M);
-                    const float* io_p = a.iobs + (size_t)j * N * N + (size_t)k2 * N + x0 + c;
-#pragma unroll
-                    for (int k1 = 0; k1 < M; ++k1) {
-                        const int pix = (k2 + R * k1) * N + x0 + c;
-                        const bool masked = a.mbits ? ((mbits >> k1) & 1u) : (a.mask[pix] != 0);
-                        if (masked) continue;
-                        const float2 av = A[i][k1], bv = u[i][k1];
-                        const float ic = cnorm(av) * invN2 + (a.bg ? __ldg(a.bg + pix) : 0.f);
-                        const float di = 2.f * (av.x * bv.x + av.y * bv.y) * invN2;
-                        const float dd = d2[i][k1] + 2.f * cnorm(bv) * invN2;
-                        const float io = fmaxf(__ldcs(io_p + (size_t)R * k1 * N), 0.f);
-                        const float ric = __fdividef(1.0f, fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
-                        const float w1 = fmaf(-io, ric, 1.f);
-                        const float q = di * ric;  // I_o dI^2 / I_c^2 = I_o q^2
-                        l1.add(w1 * di);
-                        l2.add(fmaf(w1, dd, io * q * q));
+                        const float t = 4.f * (A[i][k1].x * B[i][k1].x + A[i][k1].y * B[i][k1].y) * invN2;
+                        if constexpr (kModes)
+                            d2_s[i][k1] += t;
+                        else
+                            d2_s[i][k1] = t;
                     }
                 }
+            }
+        }
+        if constexpr (kThree) {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < S::CI1; ++i) {
+                const int w = threadIdx.x + i * kThreads;
+                if (w < C * M) {
+                    const int n1 = w / C, c = w - n1 * C;
+                    float2 vb[R];
+                    load1(vb, wb, n1, c);
+                    pass1(vb, buf1, n1, c);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < S::CI2; ++i) {
+                const int w = threadIdx.x + i * kThreads;
+                if (w < C * R) {
+                    const int k2 = w / C, c = w - k2 * C;
+                    pass2(B[i], buf1, k2, c);
+                }
+            }
+        }
+        if constexpr (kModes) {
+#pragma unroll
+            for (int i = 0; i < S::CI2; ++i)
+#pragma unroll
+                for (int k1 = 0; k1 < M; ++k1) {
+                    const float2 av = A[i][k1], bv = B[i][k1];
+                    ic_s[i][k1] += cnorm(av) * invN2;
+                    di_s[i][k1] += 2.f * (av.x * bv.x + av.y * bv.y) * invN2;
+                    d2_s[i][k1] += 2.f * cnorm(bv) * invN2;
+                }
+            if (k + 1 < K) __syncthreads();  // the buffers are free again
+        }
+    }
+    KahanF l1, l2;  // per-pixel terms in single precision (FP64 throughput is low), compensated sums
+#pragma unroll
+    for (int i = 0; i < S::CI2; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < C * R) {
+            const int k2 = w / C, c = w - k2 * C;
+            uint32_t mbits = 0u;
+            if (a.mbits) mbits = a.mbits[blockIdx.x * kThreads + threadIdx.x] >> (i * M);
+            const float* io_p = a.iobs + (size_t)j * N * N + (size_t)k2 * N + x0 + c;
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) {
+                const int pix = (k2 + R * k1) * N + x0 + c;
+                const bool masked = a.mbits ? ((mbits >> k1) & 1u) : (a.mask[pix] != 0);
+                float ic, di, dd;
+                if constexpr (kModes) {
+                    ic = ic_s[i][k1];
+                    di = di_s[i][k1];
+                    dd = d2_s[i][k1];
+                } else {
+                    const float2 av = A[i][k1], bv = B[i][k1];
+                    ic = cnorm(av) * invN2;
+                    di = 2.f * (av.x * bv.x + av.y * bv.y) * invN2;
+                    dd = 2.f * cnorm(bv) * invN2;
+                    if constexpr (kThree) dd = d2_s[i][k1] + dd;
+                }
+                if (masked) continue;
+                ic += a.bg ? __ldg(a.bg + pix) : 0.f;
+                const float io = fmaxf(__ldcs(io_p + (size_t)R * k1 * N), 0.f);
+                const float ric = __fdividef(1.0f, fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
+                const float w1 = fmaf(-io, ric, 1.f);
+                const float q = di * ric;  // I_o dI^2 / I_c^2 = I_o q^2
+                l1.add(w1 * di);
+                l2.add(fmaf(w1, dd, io * q * q));
             }
         }
     }
@@ -545,6 +618,17 @@ template <int N>
 size_t smem_col_r() {
     using S = RegShape<N>;
     return sizeof(float2) * (N + (size_t)S::C * S::P);
+}
+template <int N>
+size_t smem_col_ls_r() {
+    using S = RegShape<N>;
+    return sizeof(float2) * (N + 2 * (size_t)S::C * S::P);
+}
+inline cudaError_t ls_attrs(void (*k)(ProbArgs, int)) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e;
 }
 template <int N>
 size_t smem_row_bwd_r() {
@@ -573,7 +657,10 @@ cudaError_t set_attrs_r() {
     if ((e = cudaFuncSetAttribute(k_col_modes_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_col_modes_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_row_fwd_ls_r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_ls_r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
+    if ((e = ls_attrs(k_col_ls_r<N, false, false>))) return e;
+    if ((e = ls_attrs(k_col_ls_r<N, false, true>))) return e;
+    if ((e = ls_attrs(k_col_ls_r<N, true, false>))) return e;
+    if ((e = ls_attrs(k_col_ls_r<N, true, true>))) return e;
     if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_col_r<N, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;

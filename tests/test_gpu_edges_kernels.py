@@ -60,3 +60,43 @@ def test_position_shifts_at_edges(N, K, J):
     # 2^-21, so the shift to about 2^-21 * 0.1 * sqrt(2); 1e-5 leaves room for the condition of the 2 x 2 system
     assert np.abs(got - ref).max() < 1e-5
     pb.close()
+
+
+@pytest.mark.parametrize("N,K", [(12, 2), (32, 1), (64, 3), (80, 2), (128, 1), (128, 2), (256, 1), (256, 3), (400, 1),
+                                 (448, 2), (512, 1), (512, 3)])
+@pytest.mark.parametrize("which", ["obj", "probe", "both"])
+@pytest.mark.parametrize("J", [1, 3])
+def test_line_coeffs_every_form(N, K, which, J):
+    """L'(0) and L''(0) over the forms of the line search (two or three waves,
+    one or several modes, one frame only), with a mask, on intensities within a
+    factor of the model's so that every term is well conditioned."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + 7 * K)
+    Ho, Wo = N + 4, N + 9
+    obj, probe = crandn(rng, Ho, Wo), crandn(rng, K, N, N)
+    d_o = 0.1 * crandn(rng, Ho, Wo) if which != "probe" else None
+    d_p = 0.1 * crandn(rng, K, N, N) if which != "obj" else None
+    pos = np.stack([rng.integers(0, Ho - N + 1, J), rng.integers(0, Wo - N + 1, J)], 1).astype(np.int32)
+
+    def far(o, p):
+        return np.fft.fft2(oracle.obj_probe_to_psi(o.astype(complex), p.astype(complex), pos), norm="ortho")
+
+    A = far(obj, probe)
+    B = (0 if d_p is None else far(obj, d_p)) + (0 if d_o is None else far(d_o, probe))
+    C = 0 if d_o is None or d_p is None else far(d_o, d_p)
+    ic = (np.abs(A) ** 2).sum(1)
+    io = (ic * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+    mask = (rng.random((N, N)) < 0.1).astype(np.uint8)
+    di = 2 * (A.conj() * B).real.sum(1)
+    d2 = 2 * (np.abs(B) ** 2 + 2 * (A.conj() * C).real).sum(1)
+    t1, t2 = (1 - io / ic) * di, (1 - io / ic) * d2 + io * (di / ic) ** 2
+    good = mask == 0
+    pb = Ptycho(dev(obj), dev(probe), dev(io), pos, mask, with_psi=False)
+    got = pb.line_coeffs(None if d_o is None else dev(d_o.astype(np.complex64)),
+                         None if d_p is None else dev(d_p.astype(np.complex64))).cpu().numpy()
+    pb.close()
+    # a term's relative error: the waves' transforms (2 log2 N levels of 2^-24 relative to the rms, terms scale
+    # with |B| |A| and |B|^2) and a few roundings; 2^-18 of the sum of magnitudes covers both
+    for g, t in zip(got, (t1, t2)):
+        t = t[:, good]
+        assert abs(g - t.sum()) < 2.0 ** -18 * np.abs(t).sum(), (g, t.sum(), np.abs(t).sum())
