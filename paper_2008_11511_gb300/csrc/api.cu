@@ -162,6 +162,7 @@ struct ProbHost {
     const KernelSet* ks = nullptr;
     int L1 = 1, C2 = 1, L3 = 1;
     int B = 1;   // frames per batch
+    int Bfit = 1;  // frames that fit a lane's slice of the work stack (at most J)
     int G3 = 1;  // frame groups of row_bwd
     // object tiles met by at least one frame, with their frames (CSR, ascending j)
     std::vector<int> tile_ids, tile_ptr, tile_frames;
@@ -282,6 +283,26 @@ ptx_status check_problem(const ptx_problem& p, int idx) {
     return PTX_OK;
 }
 
+// Frames per batch when at most `most` fit: J frames in as few batches as that
+// allows (a multiple of the lanes when there are several), all of about the same
+// size, because a short last batch costs nearly a full one.  With one lane nothing
+// fills the last wave of a launch but the head of the next one, so `most` is cut
+// to whole waves of the column pass (`wave` frames each, the pass with the fewest
+// resident blocks): 1000 x 256^2 gradient, 64 -> 125 -> 112 frames per batch,
+// 831 -> 765 -> 755 us; 2500 x 128^2 LLK, 256 -> 500 -> 417 frames, 262 -> 249 ->
+// 244 us; two CG steps on 1000 x 256^2, line search in 62 -> 56 frames, 3.68 ->
+// 3.61 ms.  With two lanes, each filling the other's tails, 48 to 64 frames are
+// within 1 % (4000 x 256^2 DM cycle) and whole waves (38 frames) 2 % slower.
+size_t even_batch(size_t most, size_t J, int lanes, double wave) {
+    most = std::max<size_t>(1, std::min<size_t>(most, 32768));  // grid.y limit of the batch kernels
+    if (lanes == 1 && wave >= 1.0 && most < J && (double)most > wave)
+        most = (size_t)(std::floor((double)most / wave) * wave);
+    size_t n = (J + most - 1) / most;
+    if (n > 1) n = (n + lanes - 1) / lanes * lanes;
+    return (J + n - 1) / n;
+}
+double frames_per_wave(int per_sm, int blocks_per_frame) { return (double)per_sm * sm_count() / blocks_per_frame; }
+
 // Batches of frames: `lanes` batches are in flight at once (one per stream),
 // each with its own slice of the work-stack region of `spec_bytes`.
 
@@ -290,10 +311,8 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     const size_t frame_bytes = (size_t)p.K * p.N * p.N * sizeof(float2);
     size_t B = (spec_bytes / lanes) / 256 * 256 / frame_bytes;
     if (cap > 0 && B > (size_t)cap) B = cap;
-    if (B < 1) B = 1;
-    if (B > (size_t)p.J) B = p.J;
-    if (B > 32768) B = 32768;  // grid.y limit of the batch kernels
-    h.B = (int)B;
+    h.Bfit = (int)std::max<size_t>(1, std::min<size_t>(B, (size_t)p.J));
+    h.B = (int)even_batch(B, (size_t)p.J, lanes, frames_per_wave(h.ks->col_per_sm, p.N / h.C2));
     // frame slots G of the row-backward pass: (N / L3) row blocks x K modes x G
     // blocks, as many as are resident at once (each block loops over its
     // frames and flushes its probe sums once)
@@ -564,7 +583,7 @@ ptx_status compute_layout(std::vector<ProbHost>& probs, size_t* spec_off, size_t
         // at least the three waves per mode of one frame of the line search (more
         // than the lanes' slices hold when there is a single frame)
         const size_t frame = (size_t)h.p.K * h.p.N * h.p.N * sizeof(float2);
-        spec = std::max(spec, std::max((size_t)h.B * kDefaultLanes, (size_t)3) * frame);
+        spec = std::max(spec, std::max((size_t)h.Bfit * kDefaultLanes, (size_t)3) * frame);
         frames += (size_t)h.p.J;
     }
     *ctl_off = o;
@@ -1249,6 +1268,7 @@ ptx_status ptx_llk(ptx_handle* h, double* llk_dev, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     for (size_t pi = 0; pi < h->probs.size(); ++pi) {
         ProbHost& ph = h->probs[pi];
+        set_batch(ph, h->spec_bytes, 1, h->batch_cap, h->bwd_slots);
         const bool pdl = pass_pdl(h, ph);
         for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
             const int nb = std::min(ph.B, ph.p.J - j0);
@@ -1283,6 +1303,7 @@ ptx_status ptx_ml_grad(ptx_handle* h, void* grad_obj, void* grad_probe, double* 
     if (grad_obj) e = cudaMemsetAsync(grad_obj, 0, sizeof(float2) * (size_t)a.Ho * a.Wo, s);
     if (e == cudaSuccess && grad_probe) e = cudaMemsetAsync(grad_probe, 0, sizeof(float2) * (size_t)a.K * a.N * a.N, s);
     if (e != cudaSuccess) return cuda_fail(e, "ptx_ml_grad memset");
+    set_batch(ph, h->spec_bytes, 1, h->batch_cap, h->bwd_slots);
     const bool pdl = pass_pdl(h, ph);
     for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
         const int nb = std::min(ph.B, ph.p.J - j0);
@@ -1328,10 +1349,11 @@ ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj,
     // direction) of every mode for the register kernels, always three otherwise
     const int waves = (ph.ks->reg_lines > 0 ? ls_waves(d_obj, d_probe) : 3) * ph.p.K;
     const size_t frame_w = (size_t)waves * ph.p.N * ph.p.N * sizeof(float2);
-    size_t B = h->spec_bytes / frame_w;
-    if (B < 1) B = 1;
-    if (B > (size_t)ph.p.J) B = ph.p.J;
-    if (B > 32768) B = 32768;
+    const KernelSet* ks = ph.ks;
+    const double wave = ks->ls_per_sm
+                            ? frames_per_wave(ks->ls_per_sm(ph.p.K > 1, ls_waves(d_obj, d_probe) == 3), ph.p.N / ls_cols(ks))
+                            : 0.0;
+    const size_t B = even_batch(h->spec_bytes / frame_w, (size_t)ph.p.J, 1, wave);
     const bool pdl = pass_pdl(h, ph);
     for (int j0 = 0; j0 < ph.p.J; j0 += (int)B) {
         const int nb = std::min((int)B, ph.p.J - j0);
