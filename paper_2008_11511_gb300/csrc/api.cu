@@ -650,6 +650,12 @@ bool pass_pdl(const ptx_handle* h, const ProbHost& ph) {
     return h->pdl && !h->profiling && ph.p.nearfield <= 0.0 && !ph.p.background && use_reg_kernels(ph.ks, ph.p.K);
 }
 
+// Whether a problem's passes go out as one launch over whole frames (small
+// frames; per-kernel timing keeps the passes apart).
+bool frame_launch(const ptx_handle* h, const ProbHost& ph) {
+    return ph.ks->frame && ph.p.K == 1 && ph.p.nearfield <= 0.0 && !ph.p.background && !h->profiling;
+}
+
 // Bracket one launch with profiling events when profiling is on.
 struct ProfScope {
     ptx_handle* h;
@@ -909,7 +915,14 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
         // (one mode: with several modes the dependents waiting beside the other
         // lane's blocks cost more than they save, 20.15 -> 20.21 ms at 512^2, K = 3)
         const bool pdl = pass_pdl(h, ph) && !tc_col && ph.p.K == 1;
-        for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
+        const bool whole = frame_launch(h, ph);
+        if (whole) {
+            const int lane = next_lane;
+            next_lane = (next_lane + 1) % lanes;
+            used[lane] = true;
+            ks->frame(a, fwd_mode == X_DM ? FRAME_DM : FRAME_PHI, upd_p, lanes == 1 ? s : h->lane_stream[lane]);
+        }
+        for (int j0 = 0; j0 < ph.p.J && !whole; j0 += ph.B) {
             const int nb = std::min(ph.B, ph.p.J - j0);
             const int G = std::min(ph.G3, nb);
             const int lane = next_lane;
@@ -1270,7 +1283,9 @@ ptx_status ptx_llk(ptx_handle* h, double* llk_dev, void* stream) {
         ProbHost& ph = h->probs[pi];
         set_batch(ph, h->spec_bytes, 1, h->batch_cap, h->bwd_slots);
         const bool pdl = pass_pdl(h, ph);
-        for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
+        const bool whole = frame_launch(h, ph);
+        if (whole) ph.ks->frame(ph.args, FRAME_LLK, 0, s);
+        for (int j0 = 0; j0 < ph.p.J && !whole; j0 += ph.B) {
             const int nb = std::min(ph.B, ph.p.J - j0);
             ph.ks->row_fwd(ph.args, j0, nb, X_PHI, s, pdl && j0 > 0);
             if (ph.p.nearfield > 0.0) {

@@ -100,3 +100,46 @@ def test_line_coeffs_every_form(N, K, which, J):
     for g, t in zip(got, (t1, t2)):
         t = t[:, good]
         assert abs(g - t.sum()) < 2.0 ** -18 * np.abs(t).sum(), (g, t.sum(), np.abs(t).sum())
+
+
+@pytest.mark.parametrize("N", [32, 64])
+@pytest.mark.parametrize("J", [1, 5, 700])
+@pytest.mark.parametrize("masked", [False, True])
+def test_whole_frame_cycles(N, J, masked):
+    """Small frames whose passes are one launch: DM from a given exit wave and
+    AP against the oracle, one frame, fewer and more frames than blocks."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + J)
+    Ho, Wo = N + 23, N + 18
+    obj = (1 + 0.3 * crandn(rng, Ho, Wo)).astype(np.complex64)
+    probe = crandn(rng, 1, N, N)
+    pos = np.stack([rng.integers(0, Ho - N + 1, J), rng.integers(0, Wo - N + 1, J)], 1).astype(np.int32)
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)
+    psi = (phi * (1 + 0.1 * crandn(rng, *phi.shape))).astype(np.complex64)
+    ic = (np.abs(np.fft.fft2(phi, norm="ortho")) ** 2).sum(1)
+    io = (ic * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+    mask = (rng.random((N, N)) < 0.1).astype(np.uint8) if masked else None
+    data = oracle.Data.make(io, pos, mask)
+
+    def rel(a, b):
+        return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+    # single precision: 4 transforms of log2 N levels and a dozen roundings, each 2^-24 of the rms; the
+    # probe and object sums add J terms in FP32
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))
+    for dm in (True, False):
+        o, p = dev(obj), dev(probe)
+        pb = Ptycho(o, p, dev(io), pos, mask, psi=dev(psi))
+        l0 = float(pb.llk())
+        llk = (pb.dm(1) if dm else pb.ap(1)).cpu().numpy()
+        if dm:
+            ro, rp, rpsi, rl = oracle.dm_cycle(obj, probe, psi, data)
+        else:
+            ro, rp, rl = oracle.ap_cycle(obj, probe, data)
+        assert rel(o.cpu().numpy(), ro) < tol and rel(p.cpu().numpy(), rp) < tol
+        if dm:
+            assert rel(pb.psi.cpu().numpy(), rpsi) < tol
+        else:  # the cycle's likelihood is that of the same model waves
+            assert abs(l0 - rl) < 1e-6 * rl
+        assert abs(llk[0] - rl) < 1e-6 * abs(rl)
+        pb.close()
