@@ -167,6 +167,7 @@ struct ProbHost {
     // object tiles met by at least one frame, with their frames (CSR, ascending j)
     std::vector<int> tile_ids, tile_ptr, tile_frames;
     int ntx = 0;
+    int gather_split = 1;  // blocks per tile of the tensor-copy gather
     int tile_h = 0;  // object tile height of the gather (0: not chosen yet)
     Layout lay{};
     ProbArgs args{};
@@ -181,8 +182,9 @@ struct ProbHost {
     bool tma_gather = false;
 };
 
-// Tiles of TW x TH object pixels met by at least one frame.
-size_t active_tiles(const ptx_problem& p, const int32_t* positions, int TW, int TH) {
+// Tiles of TW x TH object pixels met by at least one frame (pairs: frames per
+// tile summed over the tiles).
+size_t active_tiles(const ptx_problem& p, const int32_t* positions, int TW, int TH, size_t* pairs = nullptr) {
     const int ntx = (p.Wo + TW - 1) / TW, nty = (p.Ho + TH - 1) / TH;
     std::vector<char> hit((size_t)ntx * nty, 0);
     for (int j = 0; j < p.J; ++j) {
@@ -192,18 +194,54 @@ size_t active_tiles(const ptx_problem& p, const int32_t* positions, int TW, int 
     }
     size_t n = 0;
     for (char v : hit) n += v;
+    if (pairs) {
+        *pairs = 0;
+        for (int j = 0; j < p.J; ++j) {
+            const int r = positions[2 * j], c = positions[2 * j + 1];
+            *pairs += (size_t)((r + p.N - 1) / TH - r / TH + 1) * ((c + p.N - 1) / TW - c / TW + 1);
+        }
+    }
     return n;
 }
 
 // Per-tile frame lists of the object gather (host, from the positions).  The
-// tile height is chosen once, at the first build: the full kObjTileH, or half
-// or a quarter of it while the object has fewer tiles than two blocks per SM
-// (a small object would otherwise leave most SMs idle).
+// tile height and the blocks per tile are chosen once, at the first build, so
+// that a small object does not leave most SMs idle.  A tile's frames are a
+// serial chain of copies: the tensor-copy gather (N >= 64) shares a tile among a
+// cluster of blocks when there are fewer than kFewTiles full tiles with at least
+// kLongChain copies each, and takes half tiles below half of that.
+// us per gather and normalisation:
+//                                 full tiles in clusters of | half tiles of
+//                                   1     2     4           |   1     2     4
+//   100 x  64^2 on  256^2 ( 64)    18    16    18           |  16    14    19
+//   150 x  64^2 on  162^2 ( 36)    52    32    23           |  46    29    19
+//   301 x 128^2 on  397^2 (169)    49    33    33           |  44    34    41
+//    97 x 192^2 on  420^2 (196)    37    27    30           |  35    29    37
+//    60 x 256^2 on  500^2 (250)    27    26    38           |  27    31    47
+//   500 x 256^2 on 1100^2          83   104   166           |  89   155   235
+// The plain gather halves the height while there are fewer tiles than two blocks
+// per SM.
+constexpr size_t kFewTiles = 250;
+constexpr size_t kLongChain = 12;
 void build_tiles(ProbHost& h, const int32_t* positions) {
     const ptx_problem& p = h.p;
     if (h.tile_h == 0) {
         h.tile_h = kObjTileH;
-        while (h.tile_h > kObjTileH / 4 && active_tiles(p, positions, kObjTileW, h.tile_h) < 2 * 152) h.tile_h /= 2;
+        if (p.N >= 64) {
+            size_t pairs = 0;
+            const size_t n = active_tiles(p, positions, kObjTileW, kObjTileH, &pairs);
+            if (n < kFewTiles && pairs * p.K >= kLongChain * n) {
+                h.gather_split = 2;
+                if (n < kFewTiles / 2) {
+                    h.tile_h = kObjTileH / 2;
+                    if (active_tiles(p, positions, kObjTileW, h.tile_h) < 100) h.gather_split = 4;
+                }
+            } else if (n < kFewTiles) {
+                h.tile_h = kObjTileH / 2;
+            }
+        } else {
+            while (h.tile_h > kObjTileH / 4 && active_tiles(p, positions, kObjTileW, h.tile_h) < 2 * 152) h.tile_h /= 2;
+        }
     }
     const int TW = kObjTileW, TH = h.tile_h;
     const int ntx = (p.Wo + TW - 1) / TW, nty = (p.Ho + TH - 1) / TH;
@@ -361,7 +399,7 @@ size_t layout_problem(ProbHost& h) {
     h.lay.llk_part = o;
     o = align_up(o + sizeof(double) * (size_t)p.J * (p.N / h.C2));
     h.lay.maxbits = o;
-    o = align_up(o + 2 * sizeof(unsigned));
+    o = align_up(o + 4 * sizeof(unsigned));
     // tile lists sized for any positions (ptx_set_positions rewrites them in place):
     // every object tile, and per frame the tiles an N x N patch can meet
     const int th = h.tile_h > 0 ? h.tile_h : kObjTileH / 4;
@@ -494,6 +532,9 @@ struct ptx_handle {
     size_t spec_bytes = 0;
     cudaStream_t lane_stream[kMaxLanes] = {};
     cudaEvent_t fork_ev = nullptr;
+    // the LLK reductions of the problems, beside their overlap updates
+    cudaStream_t llk_stream = nullptr;
+    cudaEvent_t llk_ev = nullptr;
     cudaEvent_t join_ev[kMaxLanes] = {};
     std::vector<cudaEvent_t> prob_ev;  // [problem][lane]: a problem's batches done on a lane
     // per-kernel timing (ptx_profile_enable)
@@ -682,15 +723,27 @@ struct ProfScope {
     }
 };
 
+// Blocks of k_normalise for n pixels: no more than there are pixels for.
+unsigned normalise_blocks(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 4 * 152); }
+
+// Second half of Psi2ObjProbe.  (Launched as programmatic dependents of one another these kernels' waiting
+// blocks only take the place of the lanes' blocks: 2 x 28 frames of 256^2, 113 ->
+// 118 us; six scans in one handle, 755 -> 766 us.)
 void enqueue_stages(ptx_handle* h, ProbHost& ph, int stages, cudaStream_t s) {
     const ProbArgs& a = ph.args;
+    const float ao = (float)h->alpha_obj, ap = (float)h->alpha_probe;
     if (stages & STAGE_PROBE) {
-        {
-            ProfScope ps(h, PTX_KERNEL_DEN_MAX, s);
-            k_den_max<<<2 * 152, 256, 0, s>>>(a, 0, 1);
+        if (a.K * a.N * a.N <= kProbeMax) {
+            ProfScope ps(h, PTX_KERNEL_NORMALISE, s);
+            launch_probe_norm(a, ap, s);
+        } else {
+            {
+                ProfScope ps(h, PTX_KERNEL_DEN_MAX, s);
+                k_den_max<<<2 * 152, 256, 0, s>>>(a, 0, 1);
+            }
+            ProfScope ps(h, PTX_KERNEL_NORMALISE, s);
+            k_normalise<<<normalise_blocks((size_t)a.K * a.N * a.N), 256, 0, s>>>(a, ao, ap, 0, 1);
         }
-        ProfScope ps(h, PTX_KERNEL_NORMALISE, s);
-        k_normalise<<<4 * 152, 256, 0, s>>>(a, (float)h->alpha_obj, (float)h->alpha_probe, 0, 1);
     }
     // gather and normalisation in one call: the gather also takes max D_O;
     // otherwise (accumulators summed across ranks in between) a separate pass does
@@ -698,7 +751,8 @@ void enqueue_stages(ptx_handle* h, ProbHost& ph, int stages, cudaStream_t s) {
     if ((stages & STAGE_OBJ_GATHER) && !ph.tile_ids.empty()) {
         ProfScope ps(h, PTX_KERNEL_OBJ_GATHER, s);
         if (h->tma_gather && ph.tma_gather)
-            launch_obj_gather_tma(&ph.tm_psi3, &ph.tm_probe3, a, ph.tiles, (int)ph.tile_ids.size(), fused_max ? 1 : 0, s);
+            launch_obj_gather_tma(&ph.tm_psi3, &ph.tm_probe3, a, ph.tiles, (int)ph.tile_ids.size(), ph.gather_split,
+                                  fused_max ? 1 : 0, s);
         else
             k_obj_gather<<<(unsigned)ph.tile_ids.size(), 256, 0, s>>>(a, ph.tiles, fused_max ? 1 : 0);
     }
@@ -708,7 +762,7 @@ void enqueue_stages(ptx_handle* h, ProbHost& ph, int stages, cudaStream_t s) {
             k_den_max<<<2 * 152, 256, 0, s>>>(a, 1, 0);
         }
         ProfScope ps(h, PTX_KERNEL_NORMALISE, s);
-        k_normalise<<<4 * 152, 256, 0, s>>>(a, (float)h->alpha_obj, (float)h->alpha_probe, 1, 0);
+        k_normalise<<<normalise_blocks((size_t)a.Ho * a.Wo), 256, 0, s>>>(a, ao, ap, 1, 0);
     }
 }
 
@@ -716,6 +770,10 @@ ptx_status ensure_lanes(ptx_handle* h) {
     cudaError_t e;
     if (!h->fork_ev && (e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming)) != cudaSuccess)
         return cuda_fail(e, "cudaEventCreate");
+    if (!h->llk_ev && (e = cudaEventCreateWithFlags(&h->llk_ev, cudaEventDisableTiming)) != cudaSuccess)
+        return cuda_fail(e, "cudaEventCreate");
+    if (!h->llk_stream && (e = cudaStreamCreateWithFlags(&h->llk_stream, cudaStreamNonBlocking)) != cudaSuccess)
+        return cuda_fail(e, "cudaStreamCreateWithFlags");
     while (h->prob_ev.size() < h->probs.size() * kMaxLanes) {
         cudaEvent_t ev;
         if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess)
@@ -868,6 +926,12 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
     const int lanes = h->profiling ? 1 : h->lanes;  // per-kernel timing wants kernels alone
     const bool pers = h->persistent && !h->profiling && pers_eligible(h) && !(flags & PTX_UPDATE_BACKGROUND) &&
                       form == TC_NONE;
+    if (lanes > 1 && !pers) {
+        ptx_status st = ensure_lanes(h);
+        if (st != PTX_OK) return st;
+        cudaEventRecord(h->fork_ev, s);
+        for (int l = 0; l < lanes; ++l) cudaStreamWaitEvent(h->lane_stream[l], h->fork_ev, 0);
+    }
     if (pers) {
         enqueue_persistent(h, algos, init, s);
         for (int pi = 0; pi < np; ++pi) {
@@ -883,12 +947,8 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
         return PTX_OK;
     }
-    if (lanes > 1) {
-        ptx_status st = ensure_lanes(h);
-        if (st != PTX_OK) return st;
-        cudaEventRecord(h->fork_ev, s);
-        for (int l = 0; l < lanes; ++l) cudaStreamWaitEvent(h->lane_stream[l], h->fork_ev, 0);
-    }
+    // the LLK reductions: a stream of their own beside the overlap updates
+    cudaStream_t llk_s = lanes > 1 ? h->llk_stream : s;
     // lane slices of the work stack, in elements, 256-byte aligned
     const size_t slice = (h->spec_bytes / lanes) / 256 * 256 / sizeof(float2);
     int next_lane = 0;
@@ -984,20 +1044,24 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
                     cudaEvent_t ev = h->prob_ev[(size_t)pi * kMaxLanes + l];
                     cudaEventRecord(ev, h->lane_stream[l]);
                     cudaStreamWaitEvent(s, ev, 0);
+                    cudaStreamWaitEvent(llk_s, ev, 0);
                 }
         if (upd_bg) k_bg_update<<<2 * 152, 256, 0, s>>>(ph.p.background, (float*)(h->scratch + ph.lay.bg_acc),
                                                         (const uint8_t*)(h->scratch + ph.lay.mask), ph.p.N * ph.p.N,
                                                         1.0f / (float)ph.p.J);
         if (!(flags & PTX_NO_NORMALISE))
             enqueue_stages(h, ph, (upd_p ? STAGE_PROBE : 0) | (upd_o ? STAGE_OBJ_GATHER | STAGE_OBJ_NORMALISE : 0), s);
-        ProfScope ps(h, PTX_KERNEL_CYCLE_END, s);
-        k_cycle_end<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, a, pi, a.N / a.C2, pi == np - 1);
+        ProfScope ps(h, PTX_KERNEL_CYCLE_END, llk_s);
+        k_cycle_end<<<kCycleEndBlocks, 256, 0, llk_s>>>(h->ctl, a, pi, a.N / a.C2, pi == np - 1);
     }
-    if (lanes > 1)
+    if (lanes > 1) {
         for (int l = 0; l < lanes; ++l) {
             cudaEventRecord(h->join_ev[l], h->lane_stream[l]);
             cudaStreamWaitEvent(s, h->join_ev[l], 0);
         }
+        cudaEventRecord(h->llk_ev, llk_s);
+        cudaStreamWaitEvent(s, h->llk_ev, 0);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     return PTX_OK;
@@ -1476,8 +1540,6 @@ ptx_status ptx_normalise(ptx_handle* h, uint32_t flags, void* stream) {
     if (flags & PTX_UPDATE_OBJ) stages |= STAGE_OBJ_GATHER | STAGE_OBJ_NORMALISE;
     for (auto& ph : h->probs) {
         enqueue_stages(h, ph, stages, s);
-        cudaError_t e = cudaMemsetAsync(ph.args.maxbits, 0, 2 * sizeof(unsigned), s);
-        if (e != cudaSuccess) return cuda_fail(e, "ptx_normalise memset");
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ptx_normalise launch");
@@ -1747,6 +1809,8 @@ void ptx_destroy(ptx_handle* h) {
     }
     for (cudaEvent_t e : h->prob_ev) cudaEventDestroy(e);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
+    if (h->llk_ev) cudaEventDestroy(h->llk_ev);
+    if (h->llk_stream) cudaStreamDestroy(h->llk_stream);
     if (h->err_host) cudaFreeHost(h->err_host);
     delete h;
 }

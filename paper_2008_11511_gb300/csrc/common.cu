@@ -111,7 +111,9 @@ __global__ void k_den_max(ProbArgs a, int upd_obj, int upd_probe) {
 }
 
 // O <- (N_O + d_O O) / (D_O + d_O), d_O = alpha_obj max D_O (unchanged where the
-// denominator is 0); the same for each probe mode with D_P; accumulators cleared.
+// denominator is 0); the same for each probe mode with D_P; accumulators cleared,
+// and by the last block the maxima, which every block has read by then (a memset
+// node per cycle for them took 5 us of a 30 us cycle).
 __global__ void k_normalise(ProbArgs a, float alpha_obj, float alpha_probe, int upd_obj, int upd_probe) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -141,6 +143,75 @@ __global__ void k_normalise(ProbArgs a, float alpha_obj, float alpha_probe, int 
             a.acc_probe[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&a.maxbits[2], 1u) == gridDim.x - 1) {
+        if (upd_obj) a.maxbits[0] = 0u;
+        if (upd_probe) a.maxbits[1] = 0u;
+        a.maxbits[2] = 0u;
+    }
+}
+
+// The probe's max D_P and normalisation in one launch, for probes that one
+// cluster of kProbeCtas blocks holds in registers (K N^2 <= kProbeMax pixels): each
+// thread keeps its pixels' accumulators, the blocks' maxima meet through
+// distributed shared memory.  Replaces k_den_max and k_normalise, two launches
+// of 3 to 4 us that each wait for the one before (64^2: 4.0 us, 128^2: 6.5 us in
+// one; at 256^2 eight blocks take 14 us, the two launches 9).
+constexpr int kProbeCtas = 8, kProbeThreads = 512;
+static_assert(kProbeMax == 4 * kProbeCtas * kProbeThreads, "four pixels per thread at most");
+template <int Q>
+__global__ void __cluster_dims__(kProbeCtas, 1, 1) __launch_bounds__(kProbeThreads)
+    k_probe_norm(ProbArgs a, float alpha_probe) {
+    __shared__ float red[kProbeThreads / 32];
+    __shared__ float maxima[kProbeCtas];  // every block's, written by the others
+    const int n1 = a.N * a.N, n = a.K * n1;
+    const int i0 = blockIdx.x * kProbeThreads + threadIdx.x;
+    constexpr int kStep = kProbeCtas * kProbeThreads;
+    float4 v[Q];
+    float mx = 0.f;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int i = i0 + q * kStep;
+        v[q] = i < n ? a.acc_probe[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < n1) mx = fmaxf(mx, v[q].z);  // D_P is the same for every mode
+    }
+    mx = warp_max(mx);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x < kProbeCtas) {
+        float b = 0.f;
+#pragma unroll
+        for (int w = 0; w < kProbeThreads / 32; ++w) b = fmaxf(b, red[w]);
+        const unsigned local = (unsigned)__cvta_generic_to_shared(&maxima[blockIdx.x]);
+        unsigned remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(threadIdx.x));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(b) : "memory");
+    }
+    // (after this barrier no block touches another's shared memory)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    float m = 0.f;
+#pragma unroll
+    for (int c = 0; c < kProbeCtas; ++c) m = fmaxf(m, maxima[c]);
+    const float d = alpha_probe * m;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int i = i0 + q * kStep;
+        if (i >= n) continue;
+        const float den = v[q].z + d;
+        if (den > 0.f) {
+            const float2 o = a.probe[i];
+            a.probe[i] = make_float2((v[q].x + d * o.x) / den, (v[q].y + d * o.y) / den);
+        }
+        a.acc_probe[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+void launch_probe_norm(const ProbArgs& a, float alpha_probe, cudaStream_t s) {
+    const int q = (a.K * a.N * a.N + kProbeCtas * kProbeThreads - 1) / (kProbeCtas * kProbeThreads);
+    if (q <= 1)
+        k_probe_norm<1><<<kProbeCtas, kProbeThreads, 0, s>>>(a, alpha_probe);
+    else
+        k_probe_norm<4><<<kProbeCtas, kProbeThreads, 0, s>>>(a, alpha_probe);
 }
 
 __device__ double block_reduce_llk(const double* part, size_t n) {
@@ -186,8 +257,6 @@ __global__ void k_cycle_end(Ctl* ctl, ProbArgs a, int p, int nparts_per_frame, i
     const double r = block_reduce_llk(ctl->l2, gridDim.x);
     if (threadIdx.x == 0) {
         if (ctl->llk_out) ctl->llk_out[(size_t)ctl->cycle * ctl->nprob + p] = r;
-        a.maxbits[0] = 0u;
-        a.maxbits[1] = 0u;
         ctl->ticket = 0u;
         if (last_problem) ctl->cycle += 1;
     }

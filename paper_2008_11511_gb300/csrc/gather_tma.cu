@@ -1,5 +1,5 @@
-// Object numerator and denominator gathered per 32-column object tile (32, 16
-// or 8 rows), fed by 3D tensor copies.  For each (frame j, mode k) meeting the
+// Object numerator and denominator gathered per 32-column object tile (32 or 16
+// rows), fed by 3D tensor copies.  For each (frame j, mode k) meeting the
 // tile, the window of Psi'_jk and of P_k under the tile is one box of the
 // tile's rows x 34 columns
 // (two extra columns so that the box starts on a 16-byte boundary) copied by
@@ -19,9 +19,9 @@ namespace {
 
 constexpr int kT = 32;             // tile width (kObjTileW == 32)
 constexpr int kBoxW = kT + 2;      // 34 columns: 272 bytes per box row
-constexpr int kStages = 4;
 constexpr int kConsumers = 8;      // warps
-// one box: kRows rows of the tile (32, 16 or 8)
+constexpr int kStages = 4;
+// one box: kRows rows of the tile (32 or 16)
 template <int kRows>
 __host__ __device__ constexpr size_t box_bytes() { return sizeof(float2) * kBoxW * kRows; }
 
@@ -60,6 +60,19 @@ __device__ __forceinline__ void load_3d(uint32_t dst, const CUtensorMap* map, in
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, unsigned rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void flag_error(int* flag) {
     if (flag) {
         *(volatile int*)flag = 1;
@@ -78,7 +91,9 @@ __device__ __forceinline__ void box_origin(int2 p, int y0, int tx, int& xs, int&
 
 }  // namespace
 
-template <int kRows>
+// kSplit: a cluster of blocks shares the tile, each taking a run of its frames;
+// rank 0 adds the others' sums in rank order and writes the tile.
+template <int kRows, bool kSplit>
 __global__ void __launch_bounds__(32 * (kConsumers + 1), 2)
     k_obj_gather_t(const __grid_constant__ CUtensorMap tm_psi, const __grid_constant__ CUtensorMap tm_probe, ProbArgs a,
                    TileLists tl, int fuse_max) {
@@ -92,11 +107,21 @@ __global__ void __launch_bounds__(32 * (kConsumers + 1), 2)
     // column offset (0 or 1) of each stage's window, written by the producer
     // before its arrival on the stage's full barrier
     __shared__ int stage_off[kStages];
-    const int t = blockIdx.x;
+    unsigned rank = 0, ranks = 1;
+    if constexpr (kSplit) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(ranks));
+    }
+    const int t = blockIdx.x / ranks;
     const int tid = tl.tile_ids[t];
     const int ty = tid / tl.ntx, tx = tid - ty * tl.ntx;
     const int K = a.K;
-    const int f0 = tl.tile_ptr[t], f1 = tl.tile_ptr[t + 1];
+    int f0 = tl.tile_ptr[t], f1 = tl.tile_ptr[t + 1];
+    if constexpr (kSplit) {
+        const int n = f1 - f0;
+        f1 = f0 + (int)((long long)n * (rank + 1) / ranks);
+        f0 += (int)((long long)n * rank / ranks);
+    }
     const int nitems = (f1 - f0) * K;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -152,6 +177,11 @@ __global__ void __launch_bounds__(32 * (kConsumers + 1), 2)
             for (int q = (it > kStages ? it - kStages : 0); q < it; ++q)
                 bar_wait(s_u32(&full[q % kStages]), (q / kStages) & 1);
         }
+        if constexpr (kSplit) {  // every thread of the cluster meets both barriers
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
         return;
     }
 
@@ -186,6 +216,26 @@ __global__ void __launch_bounds__(32 * (kConsumers + 1), 2)
         if (lane == 0) bar_arrive(s_u32(&empty[s]));
     }
     if (!ok) flag_error(a.err_flag);
+    if constexpr (kSplit) {
+        // rank 0 adds the sums of the same pixels; the second barrier keeps the other
+        // blocks until it has read them
+        __shared__ float3 sums[kQ][32 * kConsumers];
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) sums[q][threadIdx.x] = make_float3(n[q].x, n[q].y, d[q]);
+        cluster_sync();
+        if (rank == 0) {
+#pragma unroll
+            for (int q = 0; q < kQ; ++q)
+                for (unsigned r = 1; r < ranks; ++r) {
+                    const uint32_t at = map_rank(s_u32(&sums[q][threadIdx.x]), r);
+                    n[q].x += ld_cluster(at);
+                    n[q].y += ld_cluster(at + 4);
+                    d[q] += ld_cluster(at + 8);
+                }
+        }
+        cluster_sync();
+        if (rank != 0) return;
+    }
     const int x = tx * kT + lane;
     float dmax = 0.f;
     if (x < a.Wo) {
@@ -206,30 +256,55 @@ __global__ void __launch_bounds__(32 * (kConsumers + 1), 2)
 }
 
 template <int kRows>
-constexpr size_t gather_smem() { return kStages * 2 * box_bytes<kRows>() + 2 * kStages * sizeof(uint64_t); }
+constexpr size_t gather_smem() {
+    return kStages * (2 * box_bytes<kRows>() + 2 * sizeof(uint64_t));
+}
 
-cudaError_t set_attrs_gather_tma() {
-    cudaError_t e = cudaFuncSetAttribute(k_obj_gather_t<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gather_smem<32>());
+template <int kRows>
+cudaError_t set_attrs_rows() {
+    cudaError_t e = cudaFuncSetAttribute(k_obj_gather_t<kRows, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gather_smem<kRows>());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_obj_gather_t<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gather_smem<16>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_obj_gather_t<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gather_smem<8>());
+        e = cudaFuncSetAttribute(k_obj_gather_t<kRows, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)gather_smem<kRows>());
     return e;
+}
+cudaError_t set_attrs_gather_tma() {
+    const cudaError_t e = set_attrs_rows<32>();
+    return e == cudaSuccess ? set_attrs_rows<16>() : e;
+}
+
+template <int kRows>
+void launch_rows(const CUtensorMap& mp, const CUtensorMap& mq, const ProbArgs& a, const TileLists& tl, int ntiles,
+                 int split, int fuse_max, cudaStream_t s) {
+    constexpr int kTh = 32 * (kConsumers + 1);
+    if (split == 1) {
+        k_obj_gather_t<kRows, false><<<ntiles, kTh, gather_smem<kRows>(), s>>>(mp, mq, a, tl, fuse_max);
+        return;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ntiles * split);
+    cfg.blockDim = dim3(kTh);
+    cfg.dynamicSmemBytes = gather_smem<kRows>();
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_obj_gather_t<kRows, true>, mp, mq, a, tl, fuse_max);
 }
 
 // tl.th selects the instantiation; the tensor maps' boxes are 34 x tl.th
 void launch_obj_gather_tma(const void* tm_psi, const void* tm_probe, const ProbArgs& a, const TileLists& tl,
-                           int ntiles, int fuse_max, cudaStream_t s) {
+                           int ntiles, int split, int fuse_max, cudaStream_t s) {
     const CUtensorMap& mp = *(const CUtensorMap*)tm_psi;
     const CUtensorMap& mq = *(const CUtensorMap*)tm_probe;
-    constexpr int kTh = 32 * (kConsumers + 1);
-    if (tl.th == 8)
-        k_obj_gather_t<8><<<ntiles, kTh, gather_smem<8>(), s>>>(mp, mq, a, tl, fuse_max);
-    else if (tl.th == 16)
-        k_obj_gather_t<16><<<ntiles, kTh, gather_smem<16>(), s>>>(mp, mq, a, tl, fuse_max);
+    if (tl.th == 16)
+        launch_rows<16>(mp, mq, a, tl, ntiles, split, fuse_max, s);
     else
-        k_obj_gather_t<32><<<ntiles, kTh, gather_smem<32>(), s>>>(mp, mq, a, tl, fuse_max);
+        launch_rows<32>(mp, mq, a, tl, ntiles, split, fuse_max, s);
 }
 
 }  // namespace ptx

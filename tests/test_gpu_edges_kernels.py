@@ -143,3 +143,28 @@ def test_whole_frame_cycles(N, J, masked):
             assert abs(l0 - rl) < 1e-6 * rl
         assert abs(llk[0] - rl) < 1e-6 * abs(rl)
         pb.close()
+
+
+# (N, K, J, side): clusters of four and two blocks per tile, one block; fewer frames than blocks of a cluster
+@pytest.mark.parametrize("N,K,J,side", [(64, 1, 3, 80), (64, 1, 150, 162), (64, 2, 100, 256), (128, 1, 90, 397),
+                                        (192, 3, 1, 420), (256, 1, 12, 900)])
+def test_object_gather_of_shared_tiles(N, K, J, side):
+    """One AP cycle: object and probe against the oracle where a tile's frames
+    are divided among the blocks of a cluster."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + J)
+    obj = (1 + 0.3 * crandn(rng, side, side)).astype(np.complex64)
+    probe = crandn(rng, K, N, N)
+    pos = rng.integers(0, side - N + 1, (J, 2)).astype(np.int32)
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)
+    ic = (np.abs(np.fft.fft2(phi, norm="ortho")) ** 2).sum(1)
+    io = (ic * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+    o, p = dev(obj), dev(probe)
+    pb = Ptycho(o, p, dev(io), pos)
+    llk = pb.ap(1).cpu().numpy()
+    ro, rp, rl = oracle.ap_cycle(obj, probe, oracle.Data.make(io, pos, None))
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
+    for a, b in ((o, ro), (p, rp)):
+        assert np.linalg.norm(a.cpu().numpy() - b) < tol * np.linalg.norm(b)
+    assert abs(llk[0] - rl) < 1e-6 * rl
+    pb.close()
