@@ -151,6 +151,7 @@ struct Layout {
     size_t pos, mask, acc_obj, acc_probe, llk_part, maxbits, tile_ids, tile_ptr, tile_frames;
     size_t cg_obj, cg_probe, ls_part, cg;  // ML conjugate-gradient state
     size_t mbits;                          // per-thread mask bits of the register column pass
+    size_t mbits_s;                        // and of the split column pass
     size_t nf_t;                           // near-field transfer factors t[k] (complex64, N)
     size_t bg_acc;                         // background update sums (float, N x N)
     size_t pos_part;                       // position-shift partial sums (double, J x bands x 5)
@@ -359,6 +360,10 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     const int resident = per_sm * sm_count();
     const int rowblk = p.N / h.L3 * p.K;
     int G = slots > 0 ? slots : resident / rowblk;
+    // split passes in several lanes: two thirds of that, leaving SMs to the other lanes' passes
+    // (4000 x 256^2 DM cycle, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us;
+    // 300 frames 270 us with 19 and 14, 273 with 10)
+    if (slots == 0 && lanes > 1 && h.ks->col_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
     if (G > h.B) G = h.B;
     if (G < 1) G = 1;
     h.G3 = G;
@@ -424,6 +429,8 @@ size_t layout_problem(ProbHost& h) {
     o = align_up(o + (8 + 3 * (size_t)kCgBlocks) * sizeof(double));  // scalars, then the dot-product partials
     h.lay.mbits = o;
     if (use_reg_kernels(h.ks, p.K)) o = align_up(o + sizeof(uint32_t) * (size_t)(p.N / h.ks->reg_cols) * kThreads);
+    h.lay.mbits_s = o;
+    if (h.ks->col_s) o = align_up(o + sizeof(uint32_t) * (size_t)h.ks->R * p.N);
     h.lay.nf_t = o;
     if (p.nearfield > 0.0) o = align_up(o + sizeof(float2) * (size_t)p.N);
     h.lay.bg_acc = o;
@@ -567,6 +574,17 @@ std::vector<uint32_t> mask_bits(const KernelSet* ks, int N, const uint8_t* mask)
     return t;
 }
 
+// Mask bits of the split column pass: bit k1 of entry k2 N + kx = mask at row
+// k2 + R k1, column kx.
+std::vector<uint32_t> mask_bits_split(const KernelSet* ks, int N, const uint8_t* mask) {
+    const int R = ks->R, M = ks->M;
+    std::vector<uint32_t> t((size_t)R * N, 0u);
+    for (size_t id = 0; id < t.size(); ++id)
+        for (int k1 = 0; k1 < M; ++k1)
+            if (mask[id + (size_t)k1 * R * N]) t[id] |= 1u << k1;
+    return t;
+}
+
 // Region of the persistent schedule's tables (after the control block): the
 // problems' arguments, the segments and batches of the work list, the item
 // counter and the per-(batch, pass) done counters, sized for batches of one
@@ -616,6 +634,7 @@ ptx_status compute_layout(std::vector<ProbHost>& probs, size_t* spec_off, size_t
         h.lay.ls_part += o;
         h.lay.cg += o;
         h.lay.mbits += o;
+        h.lay.mbits_s += o;
         h.lay.nf_t += o;
         h.lay.bg_acc += o;
         h.lay.pos_part += o;
@@ -666,6 +685,7 @@ void fill_args(ptx_handle* h, ProbHost& ph) {
     a.ls_part = (double*)(h->scratch + ph.lay.ls_part);
     a.err_flag = h->err_dev;
     a.mbits = (const uint32_t*)(h->scratch + ph.lay.mbits);
+    a.mbits_s = ph.ks->col_s ? (const uint32_t*)(h->scratch + ph.lay.mbits_s) : nullptr;
     a.nf_t = ph.p.nearfield > 0.0 ? (const float2*)(h->scratch + ph.lay.nf_t) : nullptr;
     a.bg = ph.p.background;
     a.bg_acc = nullptr;  // set only for the column passes of AP cycles that update the background
@@ -684,11 +704,26 @@ enum Stage { STAGE_PROBE = 0x100, STAGE_OBJ_GATHER = 0x200, STAGE_OBJ_NORMALISE 
 enum Algo { ALGO_AP = 0, ALGO_DM = 1 };
 
 // Whether the register batch passes of a problem go out as programmatic
-// dependents of the pass before them on the same stream: far field, no
-// background, not while profiling (whose events sit between the launches).
-// The caller launches the first forward pass of a stream plainly.
+// dependents of the pass before them on the same stream: far field without a
+// background, or the split passes, all of which wait before they touch what an
+// earlier launch writes; not while profiling (whose events sit between the
+// launches).  The caller launches the first forward pass of a stream plainly.
 bool pass_pdl(const ptx_handle* h, const ProbHost& ph) {
-    return h->pdl && !h->profiling && ph.p.nearfield <= 0.0 && !ph.p.background && use_reg_kernels(ph.ks, ph.p.K);
+    if (!h->pdl || h->profiling || !use_reg_kernels(ph.ks, ph.p.K)) return false;
+    return ph.ks->col_s || (ph.p.nearfield <= 0.0 && !ph.p.background);
+}
+
+// Whether a problem's passes are those with the column transform split between them.
+bool split_passes(const ProbHost& ph) { return ph.ks->col_s != nullptr; }
+
+// The near field's three passes between the forward and the backward row pass:
+// propagate (0), project at the detector (1), propagate back (2).
+void nearfield_part(const KernelSet* ks, const ProbArgs& a, int j0, int nb, int part, int llk_only, cudaStream_t s,
+                    bool pdl) {
+    if (part == 1)
+        ks->row_proj(a, j0, nb, llk_only, s, pdl);
+    else
+        ks->col_nf(a, nb, part == 0 ? +1 : -1, s, pdl);
 }
 
 // Whether a problem's passes go out as one launch over whole frames (small
@@ -971,10 +1006,12 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
         // another of them on the same lane (the first forward pass of a lane
         // follows event waits or the previous problem's kernels)
         const bool tc_col = form != TC_NONE && ((ph.p.N == 256 && ph.p.K == 1) || ph.p.N == 512) &&
-                            !ph.p.background;
+                            ph.p.nearfield <= 0.0 && !ph.p.background;
         // (one mode: with several modes the dependents waiting beside the other
         // lane's blocks cost more than they save, 20.15 -> 20.21 ms at 512^2, K = 3)
         const bool pdl = pass_pdl(h, ph) && !tc_col && ph.p.K == 1;
+        const bool tma_col = h->tma && ph.tma_io && ks->col_tma && ph.p.nearfield <= 0.0 && !ph.p.background;
+        const bool split = split_passes(ph) && !tc_col && !tma_col;
         const bool whole = frame_launch(h, ph);
         if (whole) {
             const int lane = next_lane;
@@ -998,22 +1035,14 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
                 if (tc_rows)
                     launch_row_fwd_tc(al, j0, nb, fwd_mode == X_DM, form, ls);
                 else
-                    ks->row_fwd(al, j0, nb, fwd_mode, ls, pdl_fwd);
+                    (split ? ks->row_fwd_s : ks->row_fwd)(al, j0, nb, fwd_mode, ls, pdl_fwd);
             }
             bool col_plain = true;  // the column pass is the register kernel (not the tensor-copy one)
             if (ph.p.nearfield > 0.0) {
                 // propagate, project at the detector, propagate back
-                {
+                for (int part = 0; part < 3; ++part) {
                     ProfScope ps(h, PTX_KERNEL_COL, ls);
-                    ks->col_nf(al, nb, +1, ls);
-                }
-                {
-                    ProfScope ps(h, PTX_KERNEL_COL, ls);
-                    ks->row_proj(al, j0, nb, 0, ls);
-                }
-                {
-                    ProfScope ps(h, PTX_KERNEL_COL, ls);
-                    ks->col_nf(al, nb, -1, ls);
+                    nearfield_part(ks, al, j0, nb, part, 0, ls, pdl);
                 }
             } else if (tc_col) {
                 ProfScope ps(h, PTX_KERNEL_COL, ls);
@@ -1021,13 +1050,13 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
             } else {
                 ProfScope ps(h, PTX_KERNEL_COL, ls);
                 CUtensorMap tm_spec;
-                const int grid = (h->tma && ph.tma_io && ks->col_tma && !ph.p.background) ? ks->col_tma_grid() : 0;
+                const int grid = tma_col ? ks->col_tma_grid() : 0;
                 if (grid > 0 && encode_2d(&tm_spec, 8, al.spec, ph.p.N, (uint64_t)ph.B * ph.p.N,
                                           (uint32_t)ks->reg_lines, (uint32_t)ph.p.N)) {
                     ks->col_tma(&tm_spec, &ph.tm_io, &ph.tm_mask, al, j0, nb, grid, ls);
                     col_plain = false;
                 } else {
-                    ks->col(al, j0, nb, COL_PROJECT, ls, pdl);
+                    (split ? ks->col_s : ks->col)(al, j0, nb, COL_PROJECT, ls, pdl);
                 }
             }
             {
@@ -1035,7 +1064,7 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
                 if (tc_rows)
                     launch_row_bwd_tc(al, j0, nb, G, upd_p ? 1 : 0, form, ls);
                 else
-                    ks->row_bwd(al, j0, nb, G, bwd_mode, 0, upd_p, ls, pdl && col_plain);
+                    (split ? ks->row_bwd_s : ks->row_bwd)(al, j0, nb, G, bwd_mode, 0, upd_p, ls, pdl && col_plain);
             }
         }
         if (lanes > 1)
@@ -1251,7 +1280,7 @@ ptx_status ptx_create(ptx_handle** out, const ptx_problem* probs, int32_t nprob,
     }
     cudaStream_t s = (cudaStream_t)stream;
     // zero everything the library owns, then copy positions and mask
-    std::vector<std::vector<uint32_t>> mbits_host(h->probs.size());
+    std::vector<std::vector<uint32_t>> mbits_host(h->probs.size()), mbits_s_host(h->probs.size());
     std::vector<std::vector<float>> nf_host(h->probs.size());
     e = cudaMemsetAsync(h->scratch, 0, spec_off, s);
     for (size_t i = 0; e == cudaSuccess && i < h->probs.size(); ++i) {
@@ -1267,6 +1296,12 @@ ptx_status ptx_create(ptx_handle** out, const ptx_problem* probs, int32_t nprob,
                 mbits_host[i] = mask_bits(ph.ks, ph.p.N, ph.p.mask);
                 e = cudaMemcpyAsync(h->scratch + ph.lay.mbits, mbits_host[i].data(), sizeof(uint32_t) * mbits_host[i].size(),
                                     cudaMemcpyHostToDevice, s);
+                if (e != cudaSuccess) break;
+            }
+            if (ph.ks->col_s) {
+                mbits_s_host[i] = mask_bits_split(ph.ks, ph.p.N, ph.p.mask);
+                e = cudaMemcpyAsync(h->scratch + ph.lay.mbits_s, mbits_s_host[i].data(),
+                                    sizeof(uint32_t) * mbits_s_host[i].size(), cudaMemcpyHostToDevice, s);
                 if (e != cudaSuccess) break;
             }
         }
@@ -1351,12 +1386,13 @@ ptx_status ptx_llk(ptx_handle* h, double* llk_dev, void* stream) {
         if (whole) ph.ks->frame(ph.args, FRAME_LLK, 0, s);
         for (int j0 = 0; j0 < ph.p.J && !whole; j0 += ph.B) {
             const int nb = std::min(ph.B, ph.p.J - j0);
-            ph.ks->row_fwd(ph.args, j0, nb, X_PHI, s, pdl && j0 > 0);
+            const bool split = split_passes(ph);
+            (split ? ph.ks->row_fwd_s : ph.ks->row_fwd)(ph.args, j0, nb, X_PHI, s, pdl && j0 > 0);
             if (ph.p.nearfield > 0.0) {
-                ph.ks->col_nf(ph.args, nb, +1, s);
-                ph.ks->row_proj(ph.args, j0, nb, 1, s);
+                nearfield_part(ph.ks, ph.args, j0, nb, 0, 1, s, pdl);
+                nearfield_part(ph.ks, ph.args, j0, nb, 1, 1, s, pdl);
             } else {
-                ph.ks->col(ph.args, j0, nb, COL_LLK, s, pdl);
+                (split ? ph.ks->col_s : ph.ks->col)(ph.args, j0, nb, COL_LLK, s, pdl);
             }
         }
         k_llk_reduce<<<1, 1024, 0, s>>>(ph.args, ph.p.N / ph.C2, llk_dev + pi);
@@ -1386,10 +1422,11 @@ ptx_status ptx_ml_grad(ptx_handle* h, void* grad_obj, void* grad_probe, double* 
     const bool pdl = pass_pdl(h, ph);
     for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
         const int nb = std::min(ph.B, ph.p.J - j0);
-        ph.ks->row_fwd(a, j0, nb, X_PHI, s, pdl && j0 > 0);
-        ph.ks->col(a, j0, nb, COL_GRAD, s, pdl);
+        const bool split = split_passes(ph);
+        (split ? ph.ks->row_fwd_s : ph.ks->row_fwd)(a, j0, nb, X_PHI, s, pdl && j0 > 0);
+        (split ? ph.ks->col_s : ph.ks->col)(a, j0, nb, COL_GRAD, s, pdl);
         if (grad_obj || grad_probe)
-            ph.ks->row_bwd(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, grad_obj != nullptr, grad_probe != nullptr, s,
+            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, grad_obj != nullptr, grad_probe != nullptr, s,
                            pdl);
     }
     if (llk_dev) k_llk_reduce<<<1, 1024, 0, s>>>(a, a.N / a.C2, llk_dev);
@@ -1421,6 +1458,10 @@ CgArgs cg_args(ptx_handle* h, ProbHost& ph) {
 // Line-search pass: L'(0), L''(0) along (dir_obj, dir_probe) into out[0..1].
 ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj, const float2* d_probe, double* out,
                                cudaStream_t s) {
+    if (!d_obj && !d_probe) {  // no direction: both are 0
+        cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(double), s);
+        return e == cudaSuccess ? PTX_OK : cuda_fail(e, "line-search memset");
+    }
     ProbArgs a = ph.args;
     a.dir_obj = d_obj;
     a.dir_probe = d_probe;
@@ -1436,8 +1477,8 @@ ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj,
     const bool pdl = pass_pdl(h, ph);
     for (int j0 = 0; j0 < ph.p.J; j0 += (int)B) {
         const int nb = std::min((int)B, ph.p.J - j0);
-        ph.ks->row_fwd_ls(a, j0, nb, pdl && j0 > 0, s);
-        ph.ks->col_ls(a, j0, nb, pdl, s);
+        ks->row_fwd_ls(a, j0, nb, pdl && j0 > 0, s);
+        ks->col_ls(a, j0, nb, pdl, s);
     }
     // partial pairs per frame: one per column block of the line-search column pass
     k_ls_reduce<<<1, 1024, 0, s>>>(a.ls_part, (size_t)ph.p.J * (ph.p.N / ls_cols(ph.ks)), out);
@@ -1459,10 +1500,11 @@ ptx_status enqueue_grad(ptx_handle* h, ProbHost& ph, float2* g_obj, float2* g_pr
     const bool pdl = pass_pdl(h, ph);
     for (int j0 = 0; j0 < ph.p.J; j0 += ph.B) {
         const int nb = std::min(ph.B, ph.p.J - j0);
-        ph.ks->row_fwd(a, j0, nb, X_PHI, s, pdl && j0 > 0);
-        ph.ks->col(a, j0, nb, COL_GRAD, s, pdl);
+        const bool split = split_passes(ph);
+        (split ? ph.ks->row_fwd_s : ph.ks->row_fwd)(a, j0, nb, X_PHI, s, pdl && j0 > 0);
+        (split ? ph.ks->col_s : ph.ks->col)(a, j0, nb, COL_GRAD, s, pdl);
         if (g_obj || g_probe)
-            ph.ks->row_bwd(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, g_obj != nullptr, g_probe != nullptr, s, pdl);
+            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, g_obj != nullptr, g_probe != nullptr, s, pdl);
     }
     if (llk_out) k_llk_reduce<<<1, 1024, 0, s>>>(a, a.N / a.C2, llk_out);
     e = cudaGetLastError();

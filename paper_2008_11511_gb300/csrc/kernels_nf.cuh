@@ -246,7 +246,7 @@ size_t smem_nf() {
 }
 
 template <int N>
-void launch_col_nf(const ProbArgs& a, int nb, int dir, cudaStream_t s) {
+void launch_col_nf(const ProbArgs& a, int nb, int dir, cudaStream_t s, bool) {
     if constexpr (Plan<N>::M > 1) {
         dim3 grid(N / RegShape<N>::L, nb);
         if (dir < 0)
@@ -256,7 +256,7 @@ void launch_col_nf(const ProbArgs& a, int nb, int dir, cudaStream_t s) {
     }
 }
 template <int N>
-void launch_row_proj(const ProbArgs& a, int j0, int nb, int llk_only, cudaStream_t s) {
+void launch_row_proj(const ProbArgs& a, int j0, int nb, int llk_only, cudaStream_t s, bool) {
     if constexpr (Plan<N>::M > 1) {
         dim3 grid(N / RegShape<N>::L, nb);
         if (!llk_only && !a.bg)

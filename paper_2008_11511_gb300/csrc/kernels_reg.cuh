@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_mod
                     f = masked ? 0.f : (ratio - 1.0f) * invN2;
                 } else {
                     if (!masked) llk += llk_term_fast(ic, io);
-                    f = masked ? 0.f : 2.0f * (1.0f - __fdividef(fmaxf(io, 0.f), fmaxf(ic, 1e-30f))) * invN2;
+                    f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
                 }
                 ic_r[i][k1] = f;
             }
@@ -356,6 +356,28 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_r(ProbArgs a, int j0, i
 // Row pass: grid (N / L, frames in batch, waves x K), blockIdx.z = wave * K +
 // mode (waves 0: A, 1: B, 2: C); row transforms into spec[b][wave][mode].
 // ---------------------------------------------------------------------------
+// The products a wave is the sum of: p o (+ p2 o2).  As pointers, so that the
+// row passes load every wave as the cycle's forward pass loads P O.
+struct LsWave {
+    const float2 *p, *o, *p2, *o2;
+};
+__device__ __forceinline__ LsWave ls_wave(const ProbArgs& a, int wave) {
+    LsWave w = {a.probe, a.obj, nullptr, nullptr};
+    if (wave == 2) {
+        w.p = a.dir_probe;
+        w.o = a.dir_obj;
+    } else if (wave == 1 && a.dir_obj) {  // dO P (+ dP O)
+        w.o = a.dir_obj;
+        if (a.dir_probe) {
+            w.p2 = a.dir_probe;
+            w.o2 = a.obj;
+        }
+    } else if (wave == 1) {
+        w.p = a.dir_probe;
+    }
+    return w;
+}
+
 template <int N>
 __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls_r(ProbArgs a, int j0) {
     using S = RegShape<N>;
@@ -368,6 +390,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
     const int y0 = blockIdx.x * L;
     const int b = blockIdx.y;
     const int wave = blockIdx.z / a.K, k = blockIdx.z - wave * a.K;
+    const LsWave w0 = ls_wave(a, wave);
     const int2 p = a.pos[j0 + b];
     __syncthreads();
 #pragma unroll
@@ -380,19 +403,10 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_ls
             const size_t oi = (size_t)(p.x + y) * a.Wo + p.y + n1;
             float2 v[R];
 #pragma unroll
-            for (int n2 = 0; n2 < R; ++n2) {
-                const size_t pk = pi + M * n2, ok = oi + M * n2;
-                float2 x;
-                if (wave == 0) {
-                    x = cmul(__ldg(a.probe + pk), __ldg(a.obj + ok));
-                } else if (wave == 1) {
-                    x = make_float2(0.f, 0.f);
-                    if (a.dir_obj) x = cmul(__ldg(a.probe + pk), __ldg(a.dir_obj + ok));
-                    if (a.dir_probe) x = cadd(x, cmul(__ldg(a.dir_probe + pk), __ldg(a.obj + ok)));
-                } else {
-                    x = cmul(__ldg(a.dir_probe + pk), __ldg(a.dir_obj + ok));
-                }
-                v[n2] = x;
+            for (int n2 = 0; n2 < R; ++n2) v[n2] = cmul(__ldg(w0.p + pi + M * n2), __ldg(w0.o + oi + M * n2));
+            if (w0.p2) {
+#pragma unroll
+                for (int n2 = 0; n2 < R; ++n2) v[n2] = cadd(v[n2], cmul(__ldg(w0.p2 + pi + M * n2), __ldg(w0.o2 + oi + M * n2)));
             }
             Dft<R, -1>::run(v);
             float2* o = buf + line * P + n1;
@@ -451,7 +465,7 @@ __global__ void __launch_bounds__(kThreads, (ls_min_blocks<N, kModes, kThree>())
     constexpr int R = S::R, M = S::M, C = S::C, P = S::P;
     constexpr int kWaves = kThree ? 3 : 2;
     extern __shared__ __align__(16) float2 sm[];
-    __shared__ double red_s[kThreads / 32];
+    __shared__ double red_s[2][kThreads];
     float2* tw = sm;
     float2* buf0 = sm + N;
     float2* buf1 = buf0 + C * P;
@@ -594,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, (ls_min_blocks<N, kModes, kThree>())
                 if (masked) continue;
                 ic += a.bg ? __ldg(a.bg + pix) : 0.f;
                 const float io = fmaxf(__ldcs(io_p + (size_t)R * k1 * N), 0.f);
-                const float ric = __fdividef(1.0f, fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
+                const float ric = rcp_ftz(fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
                 const float w1 = fmaf(-io, ric, 1.f);
                 const float q = di * ric;  // I_o dI^2 / I_c^2 = I_o q^2
                 l1.add(w1 * di);
@@ -602,14 +616,7 @@ __global__ void __launch_bounds__(kThreads, (ls_min_blocks<N, kModes, kThree>())
             }
         }
     }
-    const double t1 = block_sum_double<kThreads>(l1.value(), red_s);
-    __syncthreads();
-    const double t2 = block_sum_double<kThreads>(l2.value(), red_s);
-    if (threadIdx.x == 0) {
-        double* out = a.ls_part + 2 * ((size_t)j * gridDim.x + blockIdx.x);
-        out[0] = t1;
-        out[1] = t2;
-    }
+    block_sum_pair<kThreads>(l1.value(), l2.value(), red_s, a.ls_part + 2 * ((size_t)j * gridDim.x + blockIdx.x));
 }
 
 template <int N>
@@ -639,6 +646,14 @@ size_t smem_row_bwd_r() {
 }
 
 template <int N>
+cudaError_t set_attrs_ls() {
+    cudaError_t e = cudaFuncSetAttribute(k_row_fwd_ls_r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess) e = ls_attrs(k_col_ls_r<N, false, false>);
+    if (e == cudaSuccess) e = ls_attrs(k_col_ls_r<N, false, true>);
+    if (e == cudaSuccess) e = ls_attrs(k_col_ls_r<N, true, false>);
+    return e == cudaSuccess ? ls_attrs(k_col_ls_r<N, true, true>) : e;
+}
+template <int N>
 cudaError_t set_attrs_r() {
     cudaError_t e;
     const int mx = 200 * 1024;
@@ -656,11 +671,6 @@ cudaError_t set_attrs_r() {
     if ((e = cudaFuncSetAttribute(k_col_modes_r<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
     if ((e = cudaFuncSetAttribute(k_col_modes_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_col_modes_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_fwd_ls_r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = ls_attrs(k_col_ls_r<N, false, false>))) return e;
-    if ((e = ls_attrs(k_col_ls_r<N, false, true>))) return e;
-    if ((e = ls_attrs(k_col_ls_r<N, true, false>))) return e;
-    if ((e = ls_attrs(k_col_ls_r<N, true, true>))) return e;
     if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
     if ((e = cudaFuncSetAttribute(k_col_r<N, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;

@@ -1,0 +1,689 @@
+// Passes of the far-field cycle with the column transform split between them.
+//
+// A column of N = R M pixels needs two factors, an R-point one over the rows
+// n1 + M n2 (n2 < R) and an M-point one over n1.  A row-pass block that holds
+// the R rows n1 + M n2 of one n1 does the first factor itself after its row
+// transforms, and the backward row pass undoes it before its own, so that the
+// column pass is left with one M-point codelet, the projection and one M-point
+// codelet on values that a single thread loads and stores: no shared memory,
+// no barrier, no twiddles, and whole rows of the stack and of the intensities per
+// warp.  The arithmetic of every value is that of the passes in kernels_reg.cuh.
+//
+// The work stack of a frame is [n1][k2][kx]: block n1 of a row pass owns R N
+// contiguous values, and the thread (k2, kx) of the column pass finds its M
+// values n1 (and its M intensities, rows k2 + R k1) at id + n1 R N, id = k2 N + kx.
+//
+// Measured at 256^2, alone, per 62 frames (kernels_reg.cuh -> here): column pass 26.9
+// -> 13.9 us (from two transposes and three barriers to none: 64 % issue active, the
+// projection's arithmetic now half of it), forward row pass 20.8 -> 21.3, backward
+// 20.7 -> 22.6 with the column factor added, near-field column pass 19.1 -> 10.7,
+// line-search column pass 49 -> 27.  In the cycle: 4000 frames, DM 3.41 -> 3.13 ms; near field,
+// 500 frames, 716 -> 630 us; gradient of 1000 frames 755 -> 685 us; two CG steps
+// 3.60 -> 2.85 ms; three-mode CG step of 150 frames 944 -> 854 us.  The passes of
+// kernels_reg.cuh keep the other sizes and, at 256^2, the stack order that the
+// tensor-core, tensor-copy and persistent forms and ptx_llk_static work in.
+#pragma once
+#include "kernels_reg.cuh"
+
+namespace ptx {
+
+template <int N>
+__host__ __device__ constexpr bool use_split() {
+    return N == 256;
+}
+
+template <int N>
+struct SplitShape {
+    static constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>();
+    static constexpr int I1 = (R * M + kThreads - 1) / kThreads;  // row first-factor items of a thread (and column items)
+    static constexpr int I2 = (R * R + kThreads - 1) / kThreads;  // row second-factor items
+    static constexpr int TC = R * reg_cols<N>();                  // threads of the column pass: N / C blocks per frame
+    // a row's threads in one warp for both factors: the transpose between them needs no block barrier
+    static constexpr bool kWarpRows = R == M && 32 % R == 0 && (R * R) % kThreads == 0;
+    // (blocks per SM: forward row pass with 3 / 4 / 5: DM cycle 3282 / 3220 / 3196 us; column
+    // pass with 3 / 4 / 5, the last spilling: 3278 / 3220 / 3502)
+    static constexpr int RowBlocks = M > 16 ? 2 : 5;
+    static constexpr int ColBlocks = M > 16 ? 2 : 4;
+};
+template <int N>
+__device__ __forceinline__ void split_row_sync() {
+    if constexpr (SplitShape<N>::kWarpRows)
+        __syncwarp();
+    else
+        __syncthreads();
+}
+
+// Forward: rows n1 + M n2 of one frame and mode, row transforms, first factor of
+// the column transform with its twiddles.  grid (M, frames in batch x K)
+template <int N, bool kDM>
+__global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_row_fwd_s(ProbArgs a, int j0) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;
+    float2* buf = sm + N;
+    pdl_launch_dependents();
+    load_twiddles<N>(tw);
+    const int K = a.K, n1b = blockIdx.x;
+    const int b = blockIdx.y / K, k = blockIdx.y - b * K, j = j0 + b;
+    const int2 p = a.pos[j];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < S::I1; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < R * M) {
+            const int line = w / M, n1 = w - line * M, y = n1b + M * line;
+            const float2* pr = a.probe + ((size_t)k * N + y) * N + n1;
+            const float2* ob = a.obj + (size_t)(p.x + y) * a.Wo + p.y + n1;
+            float2 q[kDM ? R : 1];
+            if constexpr (kDM) {
+                const float2* ps = a.psi + (((size_t)j * K + k) * N + y) * N + n1;
+                const uint64_t ef = policy_evict_first();
+#pragma unroll
+                for (int n2 = 0; n2 < R; ++n2) q[n2] = ld_hint(ps + M * n2, ef);
+            }
+            float2 v[R];
+#pragma unroll
+            for (int n2 = 0; n2 < R; ++n2) v[n2] = cmul(__ldg(pr + M * n2), ob[M * n2]);
+            if constexpr (kDM) {
+#pragma unroll
+                for (int n2 = 0; n2 < R; ++n2) v[n2] = make_float2(2.f * v[n2].x - q[n2].x, 2.f * v[n2].y - q[n2].y);
+            }
+            Dft<R, -1>::run(v);
+            float2* o = buf + line * P + n1;
+            o[0] = v[0];
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, -1>(tw, k2, n1));
+        }
+    }
+    split_row_sync<N>();
+#define PTX_DST (a.spec + ((size_t)blockIdx.y * M + n1b) * R * N)
+#include "body_split_tail.inc"
+#undef PTX_DST
+}
+
+// Column pass, one mode: second factor, projection and LLK (or the gradient's
+// weights), second factor of the inverse.  grid (N / C, frames in batch)
+template <int N, bool kBg, bool kCycle>
+__global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * kThreads / SplitShape<N>::TC)
+    k_col_s(ProbArgs a, int j0, int mode_arg) {
+    const int mode = kCycle ? (int)COL_PROJECT : mode_arg;
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, RN = R * N;
+    __shared__ double red_s[S::TC / 32];
+    pdl_launch_dependents();
+    const int id = blockIdx.x * S::TC + threadIdx.x;
+    const int j = j0 + blockIdx.y;
+    const float* ib = a.iobs + (size_t)j * N * N + id;
+    float io[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) io[k1] = __ldcs(ib + k1 * RN);
+    const uint32_t mbits = a.mbits_s[id];
+    float2* spec = a.spec + (size_t)blockIdx.y * N * N + id;
+    // the forward row pass that wrote the work stack may still be running
+    pdl_wait();
+    const uint64_t el = policy_evict_last();
+    float2 u[M];
+#pragma unroll
+    for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + n1 * RN, el);
+    Dft<M, -1>::run(u);
+    constexpr float invN2 = 1.0f / float(N * N);
+    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        float ic = cnorm(u[k1]) * invN2;
+        const bool masked = (mbits >> k1) & 1u;
+        if constexpr (kBg) {  // incoherent background: one more component of the model intensity
+            const int pix = id + k1 * RN;
+            ic += __ldg(a.bg + pix);
+            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
+        }
+        float f;
+        if (mode == COL_PROJECT) {
+            float ratio;
+            const float term = llk_term_ratio(ic, io[k1], ratio);
+            if (!masked) llk += term;
+            f = masked ? 0.f : (ratio - 1.0f) * invN2;
+        } else {
+            if (!masked) llk += llk_term_fast(ic, io[k1]);
+            f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io[k1], ic)) * invN2;
+        }
+        u[k1] = cscale(u[k1], f);
+    }
+    if (mode != COL_LLK) {
+        Dft<M, +1>::run(u);
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) st_hint(spec + n1 * RN, u[n1], el);
+    }
+    const double tot = block_sum_pos<S::TC>(llk, red_s);
+    if (threadIdx.x == 0) a.llk_part[(size_t)j * gridDim.x + blockIdx.x] = tot;
+}
+
+// Column pass for K > 1 modes: the thread sums |X^_k|^2 of its pixels over the
+// modes, then transforms each mode again from the stack and applies the common
+// factor: a second M-point codelet per value instead of a write and a read of
+// X^_k.  grid (N / C, frames in batch)
+template <int N, bool kCycle>
+__global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * kThreads / SplitShape<N>::TC)
+    k_col_modes_s(ProbArgs a, int j0, int mode_arg) {
+    const int mode = kCycle ? (int)COL_PROJECT : mode_arg;
+    const float* bgp = kCycle ? nullptr : a.bg;
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, RN = R * N;
+    __shared__ double red_s[S::TC / 32];
+    pdl_launch_dependents();
+    const int K = a.K;
+    const int id = blockIdx.x * S::TC + threadIdx.x;
+    const int j = j0 + blockIdx.y;
+    const uint32_t mbits = a.mbits_s[id];
+    float2* spec = a.spec + (size_t)blockIdx.y * K * N * N + id;
+    const uint64_t el = policy_evict_last();
+    float f[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) f[k1] = 0.f;
+    pdl_wait();
+    for (int k = 0; k < K; ++k) {
+        float2 u[M];
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + (size_t)k * N * N + n1 * RN, el);
+        Dft<M, -1>::run(u);
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) f[k1] += cnorm(u[k1]);
+    }
+    constexpr float invN2 = 1.0f / float(N * N);
+    const float* ib = a.iobs + (size_t)j * N * N + id;
+    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        const bool masked = (mbits >> k1) & 1u;
+        const float io = __ldcs(ib + k1 * RN);
+        float ic = f[k1] * invN2;
+        if (bgp) {
+            const int pix = id + k1 * RN;
+            ic += __ldg(bgp + pix);
+            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+        }
+        if (mode == COL_PROJECT) {
+            float ratio;
+            const float term = llk_term_ratio(ic, io, ratio);
+            if (!masked) llk += term;
+            f[k1] = masked ? 0.f : (ratio - 1.0f) * invN2;
+        } else {
+            if (!masked) llk += llk_term_fast(ic, io);
+            f[k1] = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
+        }
+    }
+    if (mode != COL_LLK) {
+        for (int k = 0; k < K; ++k) {
+            float2 u[M];
+#pragma unroll
+            for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + (size_t)k * N * N + n1 * RN, el);
+            Dft<M, -1>::run(u);
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) u[k1] = cscale(u[k1], f[k1]);
+            Dft<M, +1>::run(u);
+#pragma unroll
+            for (int n1 = 0; n1 < M; ++n1) st_hint(spec + (size_t)k * N * N + n1 * RN, u[n1], el);
+        }
+    }
+    const double tot = block_sum_pos<S::TC>(llk, red_s);
+    if (threadIdx.x == 0) a.llk_part[(size_t)j * gridDim.x + blockIdx.x] = tot;
+}
+
+// Near field: column pass of the propagator (k_col_nf's arithmetic), h or
+// conj(h) between the second factors.  grid (N / C, frames in batch)
+template <int N, int DIR>
+__global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * kThreads / SplitShape<N>::TC)
+    k_col_nf_s(ProbArgs a) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, RN = R * N;
+    pdl_launch_dependents();
+    const int id = blockIdx.x * S::TC + threadIdx.x;
+    const int k2 = id / N, kx = id - k2 * N;
+    float2* spec = a.spec + (size_t)blockIdx.y * N * N + id;
+    float2 tx = a.nf_t[kx];
+    if constexpr (DIR < 0) tx.y = -tx.y;
+    constexpr float invN2 = 1.0f / float(N * N);
+    pdl_wait();
+    const uint64_t el = policy_evict_last();
+    float2 u[M];
+#pragma unroll
+    for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + n1 * RN, el);
+    Dft<M, -1>::run(u);
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        float2 ty = __ldg(a.nf_t + k2 + R * k1);
+        if constexpr (DIR < 0) ty.y = -ty.y;
+        u[k1] = cscale(cmul(u[k1], cmul(ty, tx)), invN2);
+    }
+    Dft<M, +1>::run(u);
+#pragma unroll
+    for (int n1 = 0; n1 < M; ++n1) st_hint(spec + n1 * RN, u[n1], el);
+}
+
+// Near field: the rows n1b + M l at the detector (k_row_proj's arithmetic) between
+// the propagators' first column factors: inverse column factor, inverse rows,
+// projection and LLK, forward rows, forward column factor.  grid (M, frames in batch)
+template <int N, bool kCycle>
+__global__ void __launch_bounds__(kThreads, SplitShape<N>::ColBlocks) k_row_proj_s(ProbArgs a, int j0, int llk_only_arg) {
+    const int llk_only = kCycle ? 0 : llk_only_arg;
+    const float* bgp = kCycle ? nullptr : a.bg;
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P;
+    static_assert(S::kWarpRows && S::I2 == 1 && S::I1 == 1, "one item per thread, rows within a warp");
+    extern __shared__ __align__(16) float2 sm[];
+    __shared__ double red_s[kThreads / 32];
+    float2* tw = sm;
+    float2* buf = sm + N;
+    pdl_launch_dependents();
+    load_twiddles<N>(tw);
+    const int n1b = blockIdx.x, j = j0 + blockIdx.y;
+    const int line = threadIdx.x / R, t = threadIdx.x - line * R;  // R == M: the same row in both factors
+    const int y = n1b + M * line;
+    float2* spec = a.spec + ((size_t)blockIdx.y * M + n1b) * R * N;
+    float io[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) io[k1] = __ldcs(a.iobs + ((size_t)j * N + y) * N + t + R * k1);
+    __syncthreads();
+    pdl_wait();
+    {
+        const int kx = threadIdx.x;
+        const uint64_t el = policy_evict_last();
+        float2 v[R];
+#pragma unroll
+        for (int k2 = 0; k2 < R; ++k2) v[k2] = ld_hint(spec + k2 * N + kx, el);
+#pragma unroll
+        for (int k2 = 1; k2 < R; ++k2) v[k2] = cmul(v[k2], tw_get<N, +1>(tw, k2, n1b));
+        Dft<R, +1>::run(v);
+#pragma unroll
+        for (int l = 0; l < R; ++l) buf[l * P + kx] = v[l];
+    }
+    __syncthreads();
+    float2* o = buf + line * P;
+    float2 v[R];
+#pragma unroll
+    for (int n2 = 0; n2 < R; ++n2) v[n2] = o[t + M * n2];
+    __syncwarp();
+    Dft<R, +1>::run(v);
+    o[t] = v[0];
+#pragma unroll
+    for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1) + t] = cmul(v[k2], tw_get<N, +1>(tw, k2, t));
+    __syncwarp();
+    float2 u[M];
+#pragma unroll
+    for (int n1 = 0; n1 < M; ++n1) u[n1] = o[t * (M + 1) + n1];
+    __syncwarp();
+    Dft<M, +1>::run(u);  // the detector wave at x = t + R k1
+    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        const int pix = y * N + t + R * k1;
+        float ic = cnorm(u[k1]);
+        const bool masked = a.mask[pix] != 0;
+        if (bgp) {  // incoherent background in the detector plane
+            ic += __ldg(bgp + pix);
+            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
+        }
+        if (!masked) llk += llk_term_fast(ic, io[k1]);
+        const float f = masked ? 0.f : amp_ratio(io[k1], ic) - 1.0f;
+        u[k1] = cscale(u[k1], f);
+    }
+    const double tot = block_sum_double<kThreads>((double)llk, red_s);
+    if (threadIdx.x == 0) a.llk_part[(size_t)j * gridDim.x + blockIdx.x] = tot;
+    if (llk_only) return;
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) o[t + R * k1] = u[k1];
+    __syncwarp();
+#pragma unroll
+    for (int n2 = 0; n2 < R; ++n2) v[n2] = o[t + M * n2];
+    __syncwarp();
+    Dft<R, -1>::run(v);
+    o[t] = v[0];
+#pragma unroll
+    for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1) + t] = cmul(v[k2], tw_get<N, -1>(tw, k2, t));
+    __syncwarp();
+#define PTX_DST spec
+#include "body_split_tail.inc"
+#undef PTX_DST
+}
+
+// Line search (k_row_fwd_ls_r's waves): grid (M, frames in batch, waves x K)
+template <int N>
+__global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_row_fwd_ls_s(ProbArgs a, int j0) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;
+    float2* buf = sm + N;
+    pdl_launch_dependents();
+    load_twiddles<N>(tw);
+    const int n1b = blockIdx.x, b = blockIdx.y;
+    const int wave = blockIdx.z / a.K, k = blockIdx.z - wave * a.K;
+    const LsWave w0 = ls_wave(a, wave);
+    const int2 p = a.pos[j0 + b];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < S::I1; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < R * M) {
+            const int line = w / M, n1 = w - line * M, y = n1b + M * line;
+            const size_t pi = ((size_t)k * N + y) * N + n1;
+            const size_t oi = (size_t)(p.x + y) * a.Wo + p.y + n1;
+            float2 v[R];
+#pragma unroll
+            for (int n2 = 0; n2 < R; ++n2) v[n2] = cmul(__ldg(w0.p + pi + M * n2), __ldg(w0.o + oi + M * n2));
+            if (w0.p2) {
+#pragma unroll
+                for (int n2 = 0; n2 < R; ++n2) v[n2] = cadd(v[n2], cmul(__ldg(w0.p2 + pi + M * n2), __ldg(w0.o2 + oi + M * n2)));
+            }
+            Dft<R, -1>::run(v);
+            float2* o = buf + line * P + n1;
+            o[0] = v[0];
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, -1>(tw, k2, n1));
+        }
+    }
+    split_row_sync<N>();
+#define PTX_DST (a.spec + ((((size_t)b * gridDim.z + blockIdx.z) * M) + n1b) * R * N)
+#include "body_split_tail.inc"
+#undef PTX_DST
+}
+
+// Line search, column pass (k_col_ls_r's sums): second factors of every wave of
+// the thread's pixels.  grid (N / C, frames in batch)
+template <int N, bool kModes, bool kThree>
+__global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, kThree>() * kThreads / SplitShape<N>::TC))
+    k_col_ls_s(ProbArgs a, int j0) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, RN = R * N, kWaves = kThree ? 3 : 2;
+    __shared__ double red_s[2][S::TC];
+    pdl_launch_dependents();
+    const int K = kModes ? a.K : 1;
+    const int id = blockIdx.x * S::TC + threadIdx.x;
+    const int j = j0 + blockIdx.y;
+    constexpr float invN2 = 1.0f / float(N * N);
+    const float2* spec = a.spec + (size_t)blockIdx.y * K * kWaves * N * N + id;
+    const float* io_p = a.iobs + (size_t)j * N * N + id;
+    const uint32_t mbits = a.mbits_s[id];
+    float2 A[M], B[M];
+    float ic_s[kModes ? M : 1], di_s[kModes ? M : 1], d2_s[kModes || kThree ? M : 1];
+    if constexpr (kModes) {
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) ic_s[k1] = di_s[k1] = d2_s[k1] = 0.f;
+    }
+    auto wave = [&](float2* v, const float2* w) {
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) v[n1] = __ldcs(w + n1 * RN);
+    };
+    // the intensities come from HBM and are needed last: into L2 meanwhile
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) asm volatile("prefetch.global.L2 [%0];" ::"l"(io_p + k1 * RN));
+    }
+    pdl_wait();
+    for (int k = 0; k < K; ++k) {
+        const float2* wa = spec + (size_t)k * N * N;  // wave w of mode k: (w K + k) N^2
+        const float2* wb = wa + (size_t)K * N * N;
+        const float2* wc = wb + (size_t)K * N * N;
+        wave(A, wa);
+        wave(B, kThree ? wc : wb);
+        Dft<M, -1>::run(A);
+        Dft<M, -1>::run(B);
+        if constexpr (kThree) {
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) {
+                const float t = 4.f * (A[k1].x * B[k1].x + A[k1].y * B[k1].y) * invN2;
+                if constexpr (kModes)
+                    d2_s[k1] += t;
+                else
+                    d2_s[k1] = t;
+            }
+            wave(B, wb);
+            Dft<M, -1>::run(B);
+        }
+        if constexpr (kModes) {
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) {
+                ic_s[k1] += cnorm(A[k1]) * invN2;
+                di_s[k1] += 2.f * (A[k1].x * B[k1].x + A[k1].y * B[k1].y) * invN2;
+                d2_s[k1] += 2.f * cnorm(B[k1]) * invN2;
+            }
+        }
+    }
+    KahanF l1, l2;  // per-pixel terms in single precision, compensated sums
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        float ic, di, dd;
+        if constexpr (kModes) {
+            ic = ic_s[k1];
+            di = di_s[k1];
+            dd = d2_s[k1];
+        } else {
+            ic = cnorm(A[k1]) * invN2;
+            di = 2.f * (A[k1].x * B[k1].x + A[k1].y * B[k1].y) * invN2;
+            dd = 2.f * cnorm(B[k1]) * invN2;
+            if constexpr (kThree) dd = d2_s[k1] + dd;
+        }
+        if ((mbits >> k1) & 1u) continue;
+        ic += a.bg ? __ldg(a.bg + id + k1 * RN) : 0.f;
+        const float io = fmaxf(__ldcs(io_p + k1 * RN), 0.f);
+        const float ric = rcp_ftz(fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
+        const float w1 = fmaf(-io, ric, 1.f);
+        const float q = di * ric;  // I_o dI^2 / I_c^2 = I_o q^2
+        l1.add(w1 * di);
+        l2.add(fmaf(w1, dd, io * q * q));
+    }
+    block_sum_pair<S::TC>(l1.value(), l2.value(), red_s, a.ls_part + 2 * ((size_t)j * gridDim.x + blockIdx.x));
+}
+
+// Backward: first factor of the inverse column transform, row transforms, then
+// Psi' and the probe sums (or the gradient) as in the backward row pass of
+// kernels_reg.cuh.  grid (M, G K); blockIdx.y = slot * K + mode
+template <int N, int kForm>
+__global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, int nb, int mode_arg, int upd_obj_arg,
+                                                           int upd_probe_arg) {
+    const int mode = kForm == 1 ? (int)BWD_DM : kForm == 2 ? (int)BWD_GRAD : mode_arg;
+    const int upd_probe = kForm == 1 ? 1 : kForm == 2 ? 0 : upd_probe_arg;
+    const int upd_obj = kForm == 2 ? 1 : upd_obj_arg;
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P;
+    static_assert(S::kWarpRows && S::I2 == 1 && S::I1 == 1, "one item per thread, rows within a warp");
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;
+    float2* stage = sm + N;         // [R][N] next frame's values (cp.async)
+    float2* ostage = stage + R * N; // [R][N] next frame's object rows (cp.async)
+    float2* buf = ostage + R * N;
+    load_twiddles<N>(tw);
+    const int K = a.K, n1b = blockIdx.x;
+    const int slot = blockIdx.y / K, k = blockIdx.y - slot * K;
+    const int G = gridDim.y / K;
+    const bool acc_p = upd_probe != 0, acc_o = upd_obj != 0;
+    const bool stage_obj = mode != BWD_GRAD || acc_p;
+    const int line = threadIdx.x / R, k2t = threadIdx.x - line * R;  // R == M: the same row in both factors
+    const int y = n1b + M * line;
+    auto prefetch_spec = [&](int b) {
+        const float2* src = a.spec + (((size_t)b * K + k) * M + n1b) * R * N;
+        const uint64_t ef = policy_evict_first();  // the stack's last read
+#pragma unroll
+        for (int i = 0; i < R * N / 2 / kThreads; ++i) {
+            const int e = 2 * (threadIdx.x + i * kThreads);
+            cp_async16_hint(stage + e, src + e, ef);
+        }
+        cp_async_commit();
+    };
+    // the object rows of this warp's lines (8-byte aligned only)
+    auto prefetch_obj = [&](int b) {
+        if (stage_obj) {
+            const int2 q = a.pos[j0 + b];
+            constexpr int kLines = 32 / R;
+#pragma unroll
+            for (int l = 0; l < kLines; ++l) {
+                const int row = (threadIdx.x >> 5) * kLines + l;
+                const float2* src = a.obj + (size_t)(q.x + n1b + M * row) * a.Wo + q.y + (threadIdx.x & 31);
+                float2* dst = ostage + row * N + (threadIdx.x & 31);
+#pragma unroll
+                for (int i = 0; i < N / 32; ++i) cp_async8(dst + 32 * i, src + 32 * i);
+            }
+        }
+        cp_async_commit();
+    };
+    pdl_launch_dependents();
+    if (slot < nb) prefetch_obj(slot);
+    pdl_wait();
+    if (slot < nb) prefetch_spec(slot);
+    float2 np_r[M], pr_r[M];
+    float dp_r[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        np_r[k1] = make_float2(0.f, 0.f);
+        dp_r[k1] = 0.f;
+        pr_r[k1] = __ldg(a.probe + ((size_t)k * N + y) * N + k2t + R * k1);
+    }
+    for (int b = slot; b < nb; b += G) {
+        const int j = j0 + b;
+        const int2 p = a.pos[j];
+        cp_async_wait_all();
+        __syncthreads();
+        {  // columns: thread kx, first factor of the inverse over k2 -> rows n1b + M l
+            const int kx = threadIdx.x;
+            float2 v[R];
+            v[0] = stage[kx];
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2) v[k2] = cmul(stage[k2 * N + kx], tw_get<N, +1>(tw, k2, n1b));
+            Dft<R, +1>::run(v);
+#pragma unroll
+            for (int l = 0; l < R; ++l) buf[l * P + kx] = v[l];
+        }
+        __syncthreads();
+        if (b + G < nb) prefetch_spec(b + G);  // the stage is free again
+        {
+            const float2* src = buf + line * P + k2t;
+            float2 v[R];
+#pragma unroll
+            for (int n2 = 0; n2 < R; ++n2) v[n2] = src[M * n2];
+            __syncwarp();
+            Dft<R, +1>::run(v);
+            float2* o = buf + line * P + k2t;
+            o[0] = v[0];
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, +1>(tw, k2, k2t));
+        }
+        __syncwarp();
+        float2 u[M];
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) u[n1] = buf[line * P + k2t * (M + 1) + n1];
+        Dft<M, +1>::run(u);
+        const size_t orow = (size_t)(p.x + y) * a.Wo + p.y + k2t;
+        const float2* ob = stage_obj ? ostage + line * N + k2t : a.obj + orow;
+        float2* ps = (mode != BWD_GRAD) ? a.psi + (((size_t)j * K + k) * N + y) * N + k2t : nullptr;
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) {
+            const float2 obv = ob[R * k1];
+            float2 wv;
+            if (mode == BWD_GRAD) {
+                wv = u[k1];
+                if (acc_o) {
+                    const float2 t = cconjmul(pr_r[k1], wv);
+                    red_add_v2(a.grad_obj + orow + R * k1, t.x, t.y);
+                }
+            } else {
+                wv = cadd(cmul(pr_r[k1], obv), u[k1]);
+                __stcs(ps + R * k1, wv);
+            }
+            if (acc_p) {
+                const float2 t = cconjmul(obv, wv);
+                np_r[k1].x += t.x;
+                np_r[k1].y += t.y;
+                dp_r[k1] += cnorm(obv);
+            }
+        }
+        __syncwarp();
+        if (b + G < nb) prefetch_obj(b + G);  // this warp's object rows are free again
+    }
+    if (acc_p) {
+        const size_t pidx = ((size_t)k * N + y) * N + k2t;
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) {
+            if (mode == BWD_GRAD)
+                red_add_v2(a.grad_probe + pidx + R * k1, np_r[k1].x, np_r[k1].y);
+            else
+                red_add_v4(a.acc_probe + pidx + R * k1, np_r[k1].x, np_r[k1].y, dp_r[k1], 0.f);
+        }
+    }
+}
+
+template <int N>
+size_t smem_row_fwd_s() { return sizeof(float2) * (N + (size_t)Plan<N>::R * reg_pitch<N>()); }
+template <int N>
+size_t smem_row_bwd_s() { return sizeof(float2) * (N + 2 * (size_t)Plan<N>::R * N + (size_t)Plan<N>::R * reg_pitch<N>()); }
+
+template <int N>
+void launch_row_fwd_s(const ProbArgs& a, int j0, int nb, int mode, cudaStream_t s, bool pdl) {
+    const dim3 grid(Plan<N>::M, nb * a.K);
+    launch_dep(mode == X_DM ? k_row_fwd_s<N, true> : k_row_fwd_s<N, false>, grid, smem_row_fwd_s<N>(), s, pdl, a, j0);
+}
+template <int N>
+void launch_col_s(const ProbArgs& a, int j0, int nb, int mode, cudaStream_t s, bool pdl) {
+    const dim3 grid(N / reg_cols<N>(), nb);
+    auto k = a.K > 1 ? (mode == COL_PROJECT && !a.bg ? k_col_modes_s<N, true> : k_col_modes_s<N, false>)
+             : a.bg  ? (mode == COL_PROJECT ? k_col_s<N, true, true> : k_col_s<N, true, false>)
+                     : (mode == COL_PROJECT ? k_col_s<N, false, true> : k_col_s<N, false, false>);
+    static_assert(SplitShape<N>::TC == kThreads, "launch_dep's block size");
+    launch_dep(k, grid, 0, s, pdl, a, j0, mode);
+}
+template <int N>
+void launch_row_bwd_s(const ProbArgs& a, int j0, int nb, int G, int mode, int upd_obj, int upd_probe, cudaStream_t s,
+                      bool pdl) {
+    const dim3 grid(Plan<N>::M, G * a.K);
+    auto k = mode != BWD_GRAD && upd_probe ? k_row_bwd_s<N, 1>
+                                           : (mode == BWD_GRAD && upd_obj && !upd_probe ? k_row_bwd_s<N, 2> : k_row_bwd_s<N, 0>);
+    launch_dep(k, grid, smem_row_bwd_s<N>(), s, pdl, a, j0, nb, mode, upd_obj, upd_probe);
+}
+
+// Near field (pdl: as for the passes above) and line search.
+template <int N>
+void launch_col_nf_s(const ProbArgs& a, int nb, int dir, cudaStream_t s, bool pdl) {
+    launch_dep(dir < 0 ? k_col_nf_s<N, -1> : k_col_nf_s<N, +1>, dim3(N / reg_cols<N>(), nb), 0, s, pdl, a);
+}
+template <int N>
+void launch_row_proj_s(const ProbArgs& a, int j0, int nb, int llk_only, cudaStream_t s, bool pdl) {
+    launch_dep(!llk_only && !a.bg ? k_row_proj_s<N, true> : k_row_proj_s<N, false>, dim3(Plan<N>::M, nb), smem_row_fwd_s<N>(),
+               s, pdl, a, j0, llk_only);
+}
+template <int N>
+void launch_row_fwd_ls_s(const ProbArgs& a, int j0, int nb, int pdl, cudaStream_t s) {
+    launch_dep(k_row_fwd_ls_s<N>, dim3(Plan<N>::M, nb, ls_waves(a.dir_obj, a.dir_probe) * a.K), smem_row_fwd_s<N>(), s,
+               pdl != 0, a, j0);
+}
+template <int N>
+void launch_col_ls_s(const ProbArgs& a, int j0, int nb, int pdl, cudaStream_t s) {
+    const bool three = ls_waves(a.dir_obj, a.dir_probe) == 3;
+    auto k = a.K == 1 ? (three ? k_col_ls_s<N, false, true> : k_col_ls_s<N, false, false>)
+                      : (three ? k_col_ls_s<N, true, true> : k_col_ls_s<N, true, false>);
+    launch_dep(k, dim3(N / reg_cols<N>(), nb), 0, s, pdl != 0, a, j0);
+}
+
+template <class F>
+cudaError_t split_attrs(F f) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+template <int N>
+cudaError_t set_attrs_split() {
+    if constexpr (use_split<N>()) {
+        cudaError_t e;
+        if ((e = split_attrs(k_row_fwd_s<N, false>))) return e;
+        if ((e = split_attrs(k_row_fwd_s<N, true>))) return e;
+        if ((e = split_attrs(k_row_proj_s<N, false>))) return e;
+        if ((e = split_attrs(k_row_proj_s<N, true>))) return e;
+        if ((e = split_attrs(k_row_fwd_ls_s<N>))) return e;
+        if ((e = split_attrs(k_row_bwd_s<N, 0>))) return e;
+        if ((e = split_attrs(k_row_bwd_s<N, 1>))) return e;
+        if ((e = split_attrs(k_row_bwd_s<N, 2>))) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace ptx
