@@ -363,7 +363,10 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     // split passes in several lanes: two thirds of that, leaving SMs to the other lanes' passes
     // (4000 x 256^2 DM cycle, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us;
     // 300 frames 270 us with 19 and 14, 273 with 10)
-    if (slots == 0 && lanes > 1 && h.ks->col_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
+    if (slots == 0 && lanes > 1 && p.N == 256 && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
+    // (several modes of large frames: one slot would leave a third of the SMs with half their blocks;
+    // 300 three-mode 512^2 frames, 1 / 2 / 3 slots: 3966 / 3877 / 3893 us)
+    if (slots == 0 && G == 1 && 2 * resident >= 3 * rowblk) G = 2;
     if (G > h.B) G = h.B;
     if (G < 1) G = 1;
     h.G3 = G;
@@ -704,17 +707,17 @@ enum Stage { STAGE_PROBE = 0x100, STAGE_OBJ_GATHER = 0x200, STAGE_OBJ_NORMALISE 
 enum Algo { ALGO_AP = 0, ALGO_DM = 1 };
 
 // Whether the register batch passes of a problem go out as programmatic
-// dependents of the pass before them on the same stream: far field without a
-// background, or the split passes, all of which wait before they touch what an
-// earlier launch writes; not while profiling (whose events sit between the
-// launches).  The caller launches the first forward pass of a stream plainly.
+// dependents of the pass before them on the same stream: the far field's and the
+// split ones, all of which wait before they touch what an earlier launch of the
+// chain writes (the background changes only after the lanes have joined); not
+// while profiling (whose events sit between the launches).  The caller launches
+// the first forward pass of a stream plainly.
 bool pass_pdl(const ptx_handle* h, const ProbHost& ph) {
-    if (!h->pdl || h->profiling || !use_reg_kernels(ph.ks, ph.p.K)) return false;
-    return ph.ks->col_s || (ph.p.nearfield <= 0.0 && !ph.p.background);
+    return h->pdl && !h->profiling && use_reg_kernels(ph.ks, ph.p.K) && (ph.ks->split_nf || ph.p.nearfield <= 0.0);
 }
 
 // Whether a problem's passes are those with the column transform split between them.
-bool split_passes(const ProbHost& ph) { return ph.ks->col_s != nullptr; }
+bool split_passes(const ProbHost& ph) { return ph.ks->col_s && (ph.p.nearfield <= 0.0 || ph.ks->split_nf); }
 
 // The near field's three passes between the forward and the backward row pass:
 // propagate (0), project at the detector (1), propagate back (2).
@@ -1395,7 +1398,7 @@ ptx_status ptx_llk(ptx_handle* h, double* llk_dev, void* stream) {
                 (split ? ph.ks->col_s : ph.ks->col)(ph.args, j0, nb, COL_LLK, s, pdl);
             }
         }
-        k_llk_reduce<<<1, 1024, 0, s>>>(ph.args, ph.p.N / ph.C2, llk_dev + pi);
+        k_llk_sum<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, ph.args, ph.p.N / ph.C2, llk_dev + pi);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ptx_llk launch");
@@ -1429,7 +1432,7 @@ ptx_status ptx_ml_grad(ptx_handle* h, void* grad_obj, void* grad_probe, double* 
             (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, grad_obj != nullptr, grad_probe != nullptr, s,
                            pdl);
     }
-    if (llk_dev) k_llk_reduce<<<1, 1024, 0, s>>>(a, a.N / a.C2, llk_dev);
+    if (llk_dev) k_llk_sum<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, a, a.N / a.C2, llk_dev);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ptx_ml_grad launch");
     return PTX_OK;
@@ -1481,7 +1484,9 @@ ptx_status enqueue_line_coeffs(ptx_handle* h, ProbHost& ph, const float2* d_obj,
         ks->col_ls(a, j0, nb, pdl, s);
     }
     // partial pairs per frame: one per column block of the line-search column pass
-    k_ls_reduce<<<1, 1024, 0, s>>>(a.ls_part, (size_t)ph.p.J * (ph.p.N / ls_cols(ph.ks)), out);
+    const CgArgs c = cg_args(h, ph);
+    k_ls_reduce<<<kLsBlocks, 256, 0, s>>>(a.ls_part, (size_t)ph.p.J * (ph.p.N / ls_cols(ks)), c.cg_part,
+                                          reinterpret_cast<unsigned*>(c.cg + kCgTicket), out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "line-search launch");
     return PTX_OK;
@@ -1506,7 +1511,7 @@ ptx_status enqueue_grad(ptx_handle* h, ProbHost& ph, float2* g_obj, float2* g_pr
         if (g_obj || g_probe)
             (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, g_obj != nullptr, g_probe != nullptr, s, pdl);
     }
-    if (llk_out) k_llk_reduce<<<1, 1024, 0, s>>>(a, a.N / a.C2, llk_out);
+    if (llk_out) k_llk_sum<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, a, a.N / a.C2, llk_out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "gradient launch");
     return PTX_OK;
@@ -1544,6 +1549,7 @@ ptx_status ptx_ml_cycles(ptx_handle* h, int32_t ncycles, uint32_t flags, double*
     if (flags & PTX_ML_RESTART) {
         e = cudaMemsetAsync(c.gp_obj, 0, 2 * sizeof(float2) * c.n_obj, s);  // previous gradient and direction
         if (e == cudaSuccess) e = cudaMemsetAsync(c.gp_probe, 0, 2 * sizeof(float2) * c.n_probe, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c.cg + kCgPrev, 0, sizeof(double), s);
         if (e != cudaSuccess) return cuda_fail(e, "ML restart memset");
     }
     const int nblk = kCgBlocks;
@@ -1556,9 +1562,7 @@ ptx_status ptx_ml_cycles(ptx_handle* h, int32_t ncycles, uint32_t flags, double*
         if ((st = enqueue_grad(h, ph, uo ? c.g_obj : nullptr, up ? c.g_probe : nullptr, llk_dev ? llk_dev + cyc : nullptr,
                                s)) != PTX_OK)
             return st;
-        if ((e = cudaMemsetAsync(c.cg, 0, 8 * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "memset");
         k_cg_dots<<<nblk, 256, 0, s>>>(c);
-        k_cg_reduce<<<1, 256, 0, s>>>(c);
         k_cg_direction<<<nblk, 256, 0, s>>>(c);
         if ((st = enqueue_line_coeffs(h, ph, uo ? c.d_obj : nullptr, up ? c.d_probe : nullptr, c.cg + 3, s)) != PTX_OK)
             return st;

@@ -231,30 +231,48 @@ __device__ double block_reduce_llk(const double* part, size_t n) {
     return r;
 }
 
+// Sum over blocks: block b adds the contiguous chunk b of n values into l2[b]; the
+// last block to finish adds l2[0 .. gridDim.x) in index order, so the result does
+// not depend on the blocks' timing.  True in the last block (all threads), whose
+// thread 0 has the sum in r; the caller resets the ticket.
+__device__ bool sum_last_block(const double* part, size_t n, double* l2, unsigned* ticket, double& r) {
+    __shared__ bool is_last;
+    const size_t chunk = (n + gridDim.x - 1) / gridDim.x;
+    const size_t b0 = (size_t)blockIdx.x * chunk;
+    const size_t nb = b0 < n ? (n - b0 < chunk ? n - b0 : chunk) : 0;
+    const double s = block_reduce_llk(part + b0, nb);
+    if (threadIdx.x == 0) {
+        l2[blockIdx.x] = s;
+        __threadfence();
+        is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return false;
+    __threadfence();
+    r = block_reduce_llk(l2, gridDim.x);
+    return true;
+}
+
+// The LLK of one call (1000 x 256^2: one block 11.4 us, 64 blocks 5.7).
+__global__ void k_llk_sum(Ctl* ctl, ProbArgs a, int nparts_per_frame, double* out) {
+    double r;
+    if (!sum_last_block(a.llk_part, (size_t)a.J * nparts_per_frame, ctl->l2, &ctl->ticket, r)) return;
+    if (threadIdx.x == 0) {
+        *out = r;
+        ctl->ticket = 0u;
+    }
+}
+
+// The same in one block, for ptx_llk_static, which has no control block.
 __global__ void k_llk_reduce(ProbArgs a, int nparts_per_frame, double* out) {
     double r = block_reduce_llk(a.llk_part, (size_t)a.J * nparts_per_frame);
     if (threadIdx.x == 0) *out = r;
 }
 
-// The cycle's LLK: block b sums the contiguous chunk b of the partial sums
-// into ctl->l2[b]; the last block to finish sums l2[0 .. gridDim.x) in index
-// order, so the result does not depend on the blocks' timing.
+// The cycle's LLK, entered at the control block's cycle.
 __global__ void k_cycle_end(Ctl* ctl, ProbArgs a, int p, int nparts_per_frame, int last_problem) {
-    __shared__ bool is_last;
-    const size_t n = (size_t)a.J * nparts_per_frame;
-    const size_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const size_t b0 = (size_t)blockIdx.x * chunk;
-    const size_t nb = b0 < n ? (n - b0 < chunk ? n - b0 : chunk) : 0;
-    const double s = block_reduce_llk(a.llk_part + b0, nb);
-    if (threadIdx.x == 0) {
-        ctl->l2[blockIdx.x] = s;
-        __threadfence();
-        is_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    const double r = block_reduce_llk(ctl->l2, gridDim.x);
+    double r;
+    if (!sum_last_block(a.llk_part, (size_t)a.J * nparts_per_frame, ctl->l2, &ctl->ticket, r)) return;
     if (threadIdx.x == 0) {
         if (ctl->llk_out) ctl->llk_out[(size_t)ctl->cycle * ctl->nprob + p] = r;
         ctl->ticket = 0u;
@@ -379,11 +397,24 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// <G,G>, <G,Gp>, <Gp,Gp> over the object and probe parts: FP64 sums per block
-// into cg_part[block][0..2] (k_cg_reduce adds the blocks in index order, so the
-// result does not depend on scheduling).  kCgBlocks blocks of 256 threads.
+// A float as a double by its bits: the conversion instruction shares the FP64
+// pipe (a few lanes per clock) with the products it feeds.  Exact for zero and
+// normal values; others take the instruction.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0x7f800000u || (e == 0u && (b << 1) != 0u)) return (double)x;
+    const unsigned hi = (b & 0x80000000u) | (e == 0u ? 0u : ((b & 0x7fffffffu) >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// <G,G> and <G,Gp> over the object and probe parts into cg[0], cg[1]: FP64 sums
+// per block into cg_part, added in index order by the last block (so the result
+// does not depend on scheduling).  <Gp,Gp> is the <G,G> of the step that made Gp
+// (cg[kCgPrev], 0 after a restart) and goes to cg[2].  kCgBlocks blocks of 256 threads.
+// Bound: FP64 throughput.  1536^2 object: 68 us with conversions, three products and
+// a launch of its own (6 us) for the blocks' sums, 45 us now.
 __global__ void k_cg_dots(CgArgs c) {
-    double gg = 0.0, ggp = 0.0, gpgp = 0.0;
+    double gg = 0.0, ggp = 0.0;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t tot = c.n_obj + c.n_probe;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += stride) {
@@ -391,33 +422,33 @@ __global__ void k_cg_dots(CgArgs c) {
         const size_t k = o ? i : i - c.n_obj;
         const float2 g = o ? c.g_obj[k] : c.g_probe[k];
         const float2 q = o ? c.gp_obj[k] : c.gp_probe[k];
-        gg += (double)g.x * g.x + (double)g.y * g.y;
-        ggp += (double)g.x * q.x + (double)g.y * q.y;
-        gpgp += (double)q.x * q.x + (double)q.y * q.y;
+        const double gx = widen(g.x), gy = widen(g.y);
+        gg = fma(gx, gx, fma(gy, gy, gg));
+        ggp = fma(gx, widen(q.x), fma(gy, widen(q.y), ggp));
     }
-    __shared__ double red_s[256 / 32];
-    const double t0 = block_sum_double<256>(gg, red_s);
+    __shared__ double red_s[2][256];
+    __shared__ bool is_last;
+    block_sum_pair<256>(gg, ggp, red_s, c.cg_part + 2 * blockIdx.x);
     __syncthreads();
-    const double t1 = block_sum_double<256>(ggp, red_s);
-    __syncthreads();
-    const double t2 = block_sum_double<256>(gpgp, red_s);
+    unsigned* ticket = reinterpret_cast<unsigned*>(c.cg + kCgTicket);
     if (threadIdx.x == 0) {
-        c.cg_part[3 * blockIdx.x + 0] = t0;
-        c.cg_part[3 * blockIdx.x + 1] = t1;
-        c.cg_part[3 * blockIdx.x + 2] = t2;
+        __threadfence();
+        is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-}
-
-// cg[0..2] = sums of the kCgBlocks partials of k_cg_dots, in a fixed order.
-// One block of 256 threads.
-__global__ void k_cg_reduce(CgArgs c) {
-    __shared__ double red_s[256 / 32];
-    for (int q = 0; q < 3; ++q) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < kCgBlocks; b += 256) v += c.cg_part[3 * b + q];
-        const double t = block_sum_double<256>(v, red_s);
-        if (threadIdx.x == 0) c.cg[q] = t;
-        __syncthreads();
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    double v0 = 0.0, v1 = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) {
+        v0 += c.cg_part[2 * b];
+        v1 += c.cg_part[2 * b + 1];
+    }
+    __syncthreads();
+    block_sum_pair<256>(v0, v1, red_s, c.cg);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        c.cg[2] = c.cg[kCgPrev];
+        *ticket = 0u;
     }
 }
 
@@ -440,6 +471,7 @@ __global__ void k_cg_direction(CgArgs c) {
         *d = make_float2(fmaf(b, dv.x, -gv.x), fmaf(b, dv.y, -gv.y));
         *gp = gv;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) c.cg[kCgPrev] = c.cg[0];  // <Gp,Gp> of the next step
 }
 
 // alpha = -L'(0) / L''(0) (0 when L''(0) <= 0); O += alpha D_O, P += alpha D_P.
@@ -459,31 +491,36 @@ __global__ void k_cg_step(CgArgs c, float2* obj, float2* probe) {
     }
 }
 
-// Sum of the line-search partials (pairs) in a fixed order: out[0] = L'(0), out[1] = L''(0).
-__global__ void k_ls_reduce(const double* part, size_t nparts, double* out) {
-    __shared__ double red[2][32];
-    double a = 0.0, b = 0.0;
-    for (size_t i = threadIdx.x; i < nparts; i += blockDim.x) {
-        a += part[2 * i];
-        b += part[2 * i + 1];
+// Sum of the line-search partials (pairs) in a fixed order: out[0] = L'(0), out[1]
+// = L''(0); per block of kLsBlocks into scratch, then by the last block (one block
+// for 16000 pairs 15.4 us, kLsBlocks 6.5 us).
+__global__ void k_ls_reduce(const double* part, size_t nparts, double* scratch, unsigned* ticket, double* out) {
+    __shared__ double red_s[2][256];
+    __shared__ bool is_last;
+    const size_t chunk = (nparts + gridDim.x - 1) / gridDim.x;
+    const size_t b0 = (size_t)blockIdx.x * chunk, b1 = b0 + chunk < nparts ? b0 + chunk : nparts;
+    double v0 = 0.0, v1 = 0.0;
+    for (size_t i = b0 + threadIdx.x; i < b1; i += 256) {
+        const double2 v = reinterpret_cast<const double2*>(part)[i];
+        v0 += v.x;
+        v1 += v.y;
     }
-    a = warp_sum_d(a);
-    b = warp_sum_d(b);
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = a;
-        red[1][threadIdx.x >> 5] = b;
+    block_sum_pair<256>(v0, v1, red_s, scratch + 2 * blockIdx.x);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        a = threadIdx.x < (blockDim.x >> 5) ? red[0][threadIdx.x] : 0.0;
-        b = threadIdx.x < (blockDim.x >> 5) ? red[1][threadIdx.x] : 0.0;
-        a = warp_sum_d(a);
-        b = warp_sum_d(b);
-        if (threadIdx.x == 0) {
-            out[0] = a;
-            out[1] = b;
-        }
+    if (!is_last) return;
+    __threadfence();
+    v0 = v1 = 0.0;
+    if (threadIdx.x < gridDim.x) {
+        v0 = scratch[2 * threadIdx.x];
+        v1 = scratch[2 * threadIdx.x + 1];
     }
+    block_sum_pair<256>(v0, v1, red_s, out);
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 }  // namespace ptx

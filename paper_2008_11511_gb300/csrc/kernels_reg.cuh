@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_mod
             uint32_t mbits = 0u;
             if (a.mbits) mbits = a.mbits[blockIdx.x * kThreads + threadIdx.x] >> (i * M);
             const float* ib = a.iobs + (size_t)j * N * N + (size_t)k2 * N + x0 + c;
+            QuadAdd<M> bg_sum(a.bg_acc + (size_t)k2 * N + x0 + c, R * N);
 #pragma unroll
             for (int k1 = 0; k1 < M; ++k1) {
                 const int pix = (k2 + R * k1) * N + x0 + c;
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_mod
                 const float io = __ldcs(ib + (size_t)R * k1 * N);
                 if (bgp) {
                     ic += __ldg(bgp + pix);
-                    if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+                    if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
                 }
                 float f;
                 if (mode == COL_PROJECT) {

@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
     for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + n1 * RN, el);
     Dft<M, -1>::run(u);
     constexpr float invN2 = 1.0f / float(N * N);
+    [[maybe_unused]] QuadAdd<M> bg_sum(a.bg_acc + id, RN);
     float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
 #pragma unroll
     for (int k1 = 0; k1 < M; ++k1) {
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
         if constexpr (kBg) {  // incoherent background: one more component of the model intensity
             const int pix = id + k1 * RN;
             ic += __ldg(a.bg + pix);
-            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
+            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
         }
         float f;
         if (mode == COL_PROJECT) {
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
     }
     constexpr float invN2 = 1.0f / float(N * N);
     const float* ib = a.iobs + (size_t)j * N * N + id;
+    QuadAdd<M> bg_sum(a.bg_acc + id, RN);
     float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
 #pragma unroll
     for (int k1 = 0; k1 < M; ++k1) {
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
         if (bgp) {
             const int pix = id + k1 * RN;
             ic += __ldg(bgp + pix);
-            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
         }
         if (mode == COL_PROJECT) {
             float ratio;
