@@ -357,13 +357,18 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     // frames and flushes its probe sums once)
     int per_sm = h.ks->row_bwd_per_sm();
     if (per_sm <= 0) per_sm = 2;
-    const int resident = per_sm * sm_count();
-    const int rowblk = p.N / h.L3 * p.K;
+    int resident = per_sm * sm_count();
+    int rowblk = p.N / h.L3 * p.K;
+    if (h.ks->col_s && h.ks->M > h.ks->R) {  // k_row_bwd_s2: two blocks per SM, M of them per frame and mode
+        resident = 2 * sm_count();
+        rowblk = h.ks->M * p.K;
+    }
     int G = slots > 0 ? slots : resident / rowblk;
     // split passes in several lanes: two thirds of that, leaving SMs to the other lanes' passes
-    // (4000 x 256^2 DM cycle, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us;
-    // 300 frames 270 us with 19 and 14, 273 with 10)
-    if (slots == 0 && lanes > 1 && p.N == 256 && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
+    // (DM cycle, 4000 x 256^2, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us; 300
+    // frames 270 with 19 and 14, 273 with 10; 150 x 512^2, 9 / 6 / 4: 631 / 620 / 625; 203 x 400^2, 12 / 8 / 6:
+    // 644 / 638 / 642)
+    if (slots == 0 && lanes > 1 && h.ks->col_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
     // (several modes of large frames: one slot would leave a third of the SMs with half their blocks;
     // 300 three-mode 512^2 frames, 1 / 2 / 3 slots: 3966 / 3877 / 3893 us)
     if (slots == 0 && G == 1 && 2 * resident >= 3 * rowblk) G = 2;

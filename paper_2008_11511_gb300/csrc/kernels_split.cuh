@@ -29,6 +29,11 @@ namespace ptx {
 
 template <int N>
 __host__ __device__ constexpr bool use_split() {
+    return N == 256 || N >= 384;
+}
+// sizes whose near-field passes are split too (the row pass at the detector keeps rows in a warp)
+template <int N>
+__host__ __device__ constexpr bool use_split_nf() {
     return N == 256;
 }
 
@@ -484,9 +489,9 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, k
 template <int N, int kForm>
 __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, int nb, int mode_arg, int upd_obj_arg,
                                                            int upd_probe_arg) {
-    const int mode = kForm == 1 ? (int)BWD_DM : kForm == 2 ? (int)BWD_GRAD : mode_arg;
-    const int upd_probe = kForm == 1 ? 1 : kForm == 2 ? 0 : upd_probe_arg;
-    const int upd_obj = kForm == 2 ? 1 : upd_obj_arg;
+    const int mode = kForm == 1 ? (int)BWD_DM : kForm >= 2 ? (int)BWD_GRAD : mode_arg;
+    const int upd_probe = kForm == 1 || kForm == 3 ? 1 : kForm == 2 ? 0 : upd_probe_arg;
+    const int upd_obj = kForm >= 2 ? 1 : upd_obj_arg;
     using S = SplitShape<N>;
     constexpr int R = S::R, M = S::M, P = S::P;
     static_assert(S::kWarpRows && S::I2 == 1 && S::I1 == 1, "one item per thread, rows within a warp");
@@ -614,10 +619,231 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, i
     }
 }
 
+// Sixteen 32-bit words per thread of a warp in tensor memory, and the waits for
+// them (the warp's lanes of its quarter, columns from addr on).
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const float* v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(addr),
+        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+        "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
+        "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
+        "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// The same for the sizes whose second factor is larger than the first (M > R = 16):
+// two items of a thread per step (a column of 16 values; 16 pixels of a row), one
+// M-point codelet in between.  The probe sums of a thread's 32 pixels are 96 words:
+// in registers they would leave one block per SM, so they live in tensor memory (two
+// blocks share its 512 columns), which a warp reads and writes at its own lanes
+// without touching the shared-memory pipe that the transposes load.  Three-mode
+// 512^2 frames, per 19 frames alone: 118 us (kernels_reg.cuh), 131 with one block of 512
+// threads and register sums, 92 so; DM cycles with all split passes, kernels_reg.cuh ->
+// here: 300 x 512^2 of three modes 3.89 -> 3.65 ms, 150 x 512^2 680 -> 620 us, 200 x 448^2
+// 750 -> 650, 300 x 384^2 815 -> 700, AP of 203 x 400^2 with a background 717 -> 640.  (At
+// 256^2 the 48 words fit the registers beside staged loads: 22.6 us per 62 frames
+// there, 27 this way with three blocks per SM, more with four.)  grid (M, G K)
+constexpr uint32_t kBwdTmemCols = 256;
+template <int N, int kForm>
+__global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s2(ProbArgs a, int j0, int nb, int mode_arg, int upd_obj_arg,
+                                                            int upd_probe_arg) {
+    const int mode = kForm == 1 ? (int)BWD_DM : kForm >= 2 ? (int)BWD_GRAD : mode_arg;
+    const int upd_probe = kForm == 1 || kForm == 3 ? 1 : kForm == 2 ? 0 : upd_probe_arg;
+    const int upd_obj = kForm >= 2 ? 1 : upd_obj_arg;
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P, I = S::I1;
+    static_assert(R == 16 && BwdShape<N>::kSwap && BwdShape<N>::R == M, "the M-point factor first, 16 pixels per item");
+    static_assert(kThreads == R * R && I == 2 && 2 * 3 * 16 * I <= (int)kBwdTmemCols, "two warps per quarter of tensor memory");
+    extern __shared__ __align__(16) float2 sm[];
+    __shared__ uint32_t tmem_slot;
+    float2* tw = sm;
+    float2* buf = sm + N;
+    const int K = a.K, n1b = blockIdx.x, t = threadIdx.x, warp = t >> 5;
+    const int slot = blockIdx.y / K, k = blockIdx.y - slot * K;
+    const int G = gridDim.y / K;
+    const bool acc_p = upd_probe != 0, acc_o = upd_obj != 0;
+    load_twiddles<N>(tw);
+    uint32_t acc = 0;  // this thread's words: [item][Re N_P, Im N_P, D_P][16 pixels]
+    if (acc_p) {
+        if (warp == 0) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&tmem_slot)),
+                         "r"(kBwdTmemCols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        acc = tmem_slot + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * 48u * I;
+        const float zero[16] = {};
+#pragma unroll
+        for (int q = 0; q < 3 * I; ++q) tmem_st16(acc + 16 * q, zero);
+        tmem_wait_st();
+    } else {
+        __syncthreads();
+    }
+    // (only now: a dependent pass that waits with tensor memory of its own must not
+    // be able to take what a block of this one still needs)
+    pdl_launch_dependents();
+    pdl_wait();
+    const uint64_t ef = policy_evict_first();  // the stack's last read
+    for (int b = slot; b < nb; b += G) {
+        const int j = j0 + b;
+        const int2 p = a.pos[j];
+        const float2* src = a.spec + (((size_t)b * K + k) * M + n1b) * R * N;
+        {  // columns: first factor of the inverse over k2 -> rows n1b + M l
+            float2 v[I][R];
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const int kx = t + i * kThreads;
+#pragma unroll
+                for (int k2 = 0; k2 < R; ++k2)
+                    v[i][k2] = kx < N ? ld_hint(src + k2 * N + kx, ef) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+#pragma unroll
+                for (int k2 = 1; k2 < R; ++k2) v[i][k2] = cmul(v[i][k2], tw_get<N, +1>(tw, k2, n1b));
+                Dft<R, +1>::run(v[i]);
+            }
+            __syncthreads();  // the previous frame's rows have been read
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const int kx = t + i * kThreads;
+                if (kx < N) {
+#pragma unroll
+                    for (int l = 0; l < R; ++l) buf[l * P + kx] = v[i][l];
+                }
+            }
+        }
+        __syncthreads();
+        {  // rows: first factor, row t / R (its sixteen threads are in one warp), elements t % R + R i
+            const int n1 = t % R;
+            float2* o = buf + t / R * P + n1;
+            float2 v[M];
+#pragma unroll
+            for (int n2 = 0; n2 < M; ++n2) v[n2] = o[R * n2];
+            __syncwarp();
+            Dft<M, +1>::run(v);
+            o[0] = v[0];
+#pragma unroll
+            for (int k2 = 1; k2 < M; ++k2) o[k2 * (R + 1)] = cmul(v[k2], tw_bwd<N>(tw, k2, n1));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < I; ++i) {  // rows: second factor, pixels x0 + M k1 of row `line`
+            const int w = t + i * kThreads;
+            const bool on = w < N;
+            float tx[R], ty[R], tn[R];
+            if (on) {
+                const int line = w / M, x0 = w - line * M, y = n1b + M * line;
+                const float2* pr = a.probe + ((size_t)k * N + y) * N + x0;
+                const size_t orow = (size_t)(p.x + y) * a.Wo + p.y + x0;
+                float2* ps = (mode != BWD_GRAD) ? a.psi + (((size_t)j * K + k) * N + y) * N + x0 : nullptr;
+                float2 ob[R];
+                if (mode != BWD_GRAD || acc_p) {
+#pragma unroll
+                    for (int k1 = 0; k1 < R; ++k1) ob[k1] = a.obj[orow + M * k1];
+                }
+                float2 u[R];
+#pragma unroll
+                for (int n = 0; n < R; ++n) u[n] = buf[line * P + x0 * (R + 1) + n];
+                Dft<R, +1>::run(u);
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) {
+                    const float2 prv = __ldg(pr + M * k1);
+                    float2 wv;
+                    if (mode == BWD_GRAD) {
+                        wv = u[k1];
+                        if (acc_o) {
+                            const float2 c = cconjmul(prv, wv);
+                            red_add_v2(a.grad_obj + orow + M * k1, c.x, c.y);
+                        }
+                    } else {
+                        wv = cadd(cmul(prv, ob[k1]), u[k1]);
+                        __stcs(ps + M * k1, wv);
+                    }
+                    if (acc_p) {
+                        const float2 c = cconjmul(ob[k1], wv);
+                        tx[k1] = c.x;
+                        ty[k1] = c.y;
+                        tn[k1] = cnorm(ob[k1]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) tx[k1] = ty[k1] = tn[k1] = 0.f;
+            }
+            if (acc_p) {  // (whole warps)
+                __syncwarp();
+                float v[16];
+                const uint32_t at = acc + 48 * i;
+                tmem_ld16(at, v);
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) tx[k1] += v[k1];
+                tmem_st16(at, tx);
+                tmem_ld16(at + 16, v);
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) ty[k1] += v[k1];
+                tmem_st16(at + 16, ty);
+                tmem_ld16(at + 32, v);
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) tn[k1] += v[k1];
+                tmem_st16(at + 32, tn);
+            }
+        }
+        if (acc_p) tmem_wait_st();
+    }
+    if (acc_p) {
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            const int w = t + i * kThreads;
+            float nx[16], ny[16], dn[16];
+            tmem_ld16(acc + 48 * i, nx);
+            tmem_ld16(acc + 48 * i + 16, ny);
+            tmem_ld16(acc + 48 * i + 32, dn);
+            if (w < N) {
+                const int line = w / M, x0 = w - line * M, y = n1b + M * line;
+                const size_t pidx = ((size_t)k * N + y) * N + x0;
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) {
+                    if (mode == BWD_GRAD)
+                        red_add_v2(a.grad_probe + pidx + M * k1, nx[k1], ny[k1]);
+                    else
+                        red_add_v4(a.acc_probe + pidx + M * k1, nx[k1], ny[k1], dn[k1], 0.f);
+                }
+            }
+            __syncwarp();
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (warp == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_slot), "r"(kBwdTmemCols) : "memory");
+        }
+    }
+}
+
 template <int N>
 size_t smem_row_fwd_s() { return sizeof(float2) * (N + (size_t)Plan<N>::R * reg_pitch<N>()); }
 template <int N>
-size_t smem_row_bwd_s() { return sizeof(float2) * (N + 2 * (size_t)Plan<N>::R * N + (size_t)Plan<N>::R * reg_pitch<N>()); }
+size_t smem_row_bwd_s() {
+    constexpr size_t stages = Plan<N>::M > Plan<N>::R ? 0 : 2 * N;
+    return sizeof(float2) * (N + Plan<N>::R * (stages + reg_pitch<N>()));
+}
 
 template <int N>
 void launch_row_fwd_s(const ProbArgs& a, int j0, int nb, int mode, cudaStream_t s, bool pdl) {
@@ -633,13 +859,25 @@ void launch_col_s(const ProbArgs& a, int j0, int nb, int mode, cudaStream_t s, b
     static_assert(SplitShape<N>::TC == kThreads, "launch_dep's block size");
     launch_dep(k, grid, 0, s, pdl, a, j0, mode);
 }
+// The cycle's form (Psi' and probe sums), the gradient of the object and of both
+// parts have instantiations of their own (kForm 1, 2, 3), the rest takes its flags
+// from the arguments (0).
+template <int N, int kForm>
+void launch_row_bwd_form(const ProbArgs& a, int j0, int nb, int G, int mode, int upd_obj, int upd_probe, cudaStream_t s,
+                         bool pdl) {
+    const dim3 grid(Plan<N>::M, G * a.K);
+    if constexpr (Plan<N>::M > Plan<N>::R)
+        launch_dep(k_row_bwd_s2<N, kForm>, grid, smem_row_bwd_s<N>(), s, pdl, a, j0, nb, mode, upd_obj, upd_probe);
+    else
+        launch_dep(k_row_bwd_s<N, kForm>, grid, smem_row_bwd_s<N>(), s, pdl, a, j0, nb, mode, upd_obj, upd_probe);
+}
 template <int N>
 void launch_row_bwd_s(const ProbArgs& a, int j0, int nb, int G, int mode, int upd_obj, int upd_probe, cudaStream_t s,
                       bool pdl) {
-    const dim3 grid(Plan<N>::M, G * a.K);
-    auto k = mode != BWD_GRAD && upd_probe ? k_row_bwd_s<N, 1>
-                                           : (mode == BWD_GRAD && upd_obj && !upd_probe ? k_row_bwd_s<N, 2> : k_row_bwd_s<N, 0>);
-    launch_dep(k, grid, smem_row_bwd_s<N>(), s, pdl, a, j0, nb, mode, upd_obj, upd_probe);
+    auto f = mode != BWD_GRAD ? (upd_probe ? &launch_row_bwd_form<N, 1> : &launch_row_bwd_form<N, 0>)
+             : !upd_obj       ? &launch_row_bwd_form<N, 0>
+                              : (upd_probe ? &launch_row_bwd_form<N, 3> : &launch_row_bwd_form<N, 2>);
+    f(a, j0, nb, G, mode, upd_obj, upd_probe, s, pdl);
 }
 
 // Near field (pdl: as for the passes above) and line search.
@@ -667,7 +905,7 @@ void launch_col_ls_s(const ProbArgs& a, int j0, int nb, int pdl, cudaStream_t s)
 
 template <class F>
 cudaError_t split_attrs(F f) {
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return e;
@@ -678,12 +916,22 @@ cudaError_t set_attrs_split() {
         cudaError_t e;
         if ((e = split_attrs(k_row_fwd_s<N, false>))) return e;
         if ((e = split_attrs(k_row_fwd_s<N, true>))) return e;
-        if ((e = split_attrs(k_row_proj_s<N, false>))) return e;
-        if ((e = split_attrs(k_row_proj_s<N, true>))) return e;
         if ((e = split_attrs(k_row_fwd_ls_s<N>))) return e;
-        if ((e = split_attrs(k_row_bwd_s<N, 0>))) return e;
-        if ((e = split_attrs(k_row_bwd_s<N, 1>))) return e;
-        if ((e = split_attrs(k_row_bwd_s<N, 2>))) return e;
+        if constexpr (use_split_nf<N>()) {
+            if ((e = split_attrs(k_row_proj_s<N, false>))) return e;
+            if ((e = split_attrs(k_row_proj_s<N, true>))) return e;
+        }
+        if constexpr (Plan<N>::M > Plan<N>::R) {
+            if ((e = split_attrs(k_row_bwd_s2<N, 0>))) return e;
+            if ((e = split_attrs(k_row_bwd_s2<N, 1>))) return e;
+            if ((e = split_attrs(k_row_bwd_s2<N, 3>))) return e;
+            return split_attrs(k_row_bwd_s2<N, 2>);
+        } else {
+            if ((e = split_attrs(k_row_bwd_s<N, 0>))) return e;
+            if ((e = split_attrs(k_row_bwd_s<N, 1>))) return e;
+            if ((e = split_attrs(k_row_bwd_s<N, 3>))) return e;
+            return split_attrs(k_row_bwd_s<N, 2>);
+        }
     }
     return cudaSuccess;
 }

@@ -171,9 +171,9 @@ def test_object_gather_of_shared_tiles(N, K, J, side):
     pb.close()
 
 
-def _scan256(K, J, masked, seed):
+def _scan(N, K, J, masked, seed):
     rng = np.random.default_rng(seed)
-    N, side = 256, 256 + 37
+    side = N + 37
     obj = (1 + 0.3 * crandn(rng, side, side + 6)).astype(np.complex64)
     probe = crandn(rng, K, N, N)
     pos = np.stack([rng.integers(0, side - N + 1, J), rng.integers(0, side + 6 - N + 1, J)], 1).astype(np.int32)
@@ -186,34 +186,38 @@ def _scan256(K, J, masked, seed):
 
 
 # one frame; fewer and more frames than the backward pass has slots; several modes; parts of the update left out
-@pytest.mark.parametrize("K,J,masked,upd_o,upd_p", [(1, 1, True, True, True), (1, 3, False, False, True),
-                                                    (1, 23, True, True, False), (2, 2, True, True, True),
-                                                    (3, 9, False, False, False)])
-def test_split_passes_dm_cycle(K, J, masked, upd_o, upd_p):
+@pytest.mark.parametrize("N,K,J,masked,upd_o,upd_p", [
+    (256, 1, 1, True, True, True), (256, 1, 3, False, False, True), (256, 1, 23, True, True, False),
+    (256, 2, 2, True, True, True), (256, 3, 9, False, False, False), (384, 1, 1, False, True, True),
+    (384, 2, 7, True, True, False), (400, 1, 26, True, True, True), (400, 3, 2, False, False, True),
+    (448, 1, 5, True, True, True), (512, 1, 18, False, True, True), (512, 3, 2, True, True, True),
+    (512, 2, 1, True, False, False)])
+def test_split_passes_dm_cycle(N, K, J, masked, upd_o, upd_p):
     from paper_2008_11511_gb300 import Ptycho
-    obj, probe, pos, psi, io, mask = _scan256(K, J, masked, 10 * K + J)
+    obj, probe, pos, psi, io, mask = _scan(N, K, J, masked, 10 * K + J)
     data = oracle.Data.make(io, pos, mask)
     o, p = dev(obj), dev(probe)
     pb = Ptycho(o, p, dev(io), pos, mask, psi=dev(psi))
     llk = pb.dm(1, update_obj=upd_o, update_probe=upd_p).cpu().numpy()
     ro, rp, rpsi, rl = oracle.dm_cycle(obj, probe, psi, data, update_obj=upd_o, update_probe=upd_p)
-    tol = 2.0 ** -24 * (8 * 8 + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
     for a, b in ((o, ro), (p, rp), (pb.psi, rpsi)):
         assert np.linalg.norm(a.cpu().numpy() - b) <= tol * np.linalg.norm(b)
     assert abs(llk[0] - rl) < 1e-6 * rl
     pb.close()
 
 
-@pytest.mark.parametrize("K,J,masked", [(1, 1, False), (1, 21, True), (3, 4, True)])
+@pytest.mark.parametrize("N,K,J,masked", [(256, 1, 1, False), (256, 1, 21, True), (256, 3, 4, True), (384, 1, 3, True),
+                                          (400, 2, 9, False), (448, 1, 2, True), (512, 1, 11, True), (512, 3, 2, False)])
 @pytest.mark.parametrize("parts", ["obj", "probe", "both"])
-def test_split_passes_gradient(K, J, masked, parts):
+def test_split_passes_gradient(N, K, J, masked, parts):
     from paper_2008_11511_gb300 import Ptycho
-    obj, probe, pos, _, io, mask = _scan256(K, J, masked, 20 * K + J)
+    obj, probe, pos, _, io, mask = _scan(N, K, J, masked, 20 * K + J)
     pb = Ptycho(dev(obj), dev(probe), dev(io), pos, mask, with_psi=False)
     llk, go, gp = pb.ml_grad(grad_obj=parts != "probe", grad_probe=parts != "obj")
     rl, rgo, rgp = oracle.ml_grad(obj, probe, oracle.Data.make(io, pos, mask))
     # the weights 2 (1 - I_o / I_c), |.| <= 2 here, do not amplify the waves' errors
-    tol = 2 * 2.0 ** -24 * (8 * 8 + 12 + np.sqrt(J))
+    tol = 2 * 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))
     for a, b in ((go, rgo), (gp, rgp)):
         if a is not None:
             assert np.linalg.norm(a.cpu().numpy() - b) <= tol * np.linalg.norm(b)
