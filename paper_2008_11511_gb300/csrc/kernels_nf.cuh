@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_row_pro
                 if (bgp) {  // incoherent background in the detector plane
                     const int pix = y * N + k2 + R * k1;
                     ic += __ldg(bgp + pix);
-                    if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+                    if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, quotient(io, ic));
                 }
                 if (!masked) llk += llk_term_fast(ic, io);
                 const float f = masked ? 0.f : amp_ratio(io, ic) - 1.0f;

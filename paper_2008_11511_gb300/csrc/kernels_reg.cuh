@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_mod
                 const float io = __ldcs(ib + (size_t)R * k1 * N);
                 if (bgp) {
                     ic += __ldg(bgp + pix);
-                    if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+                    if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
                 }
                 float f;
                 if (mode == COL_PROJECT) {

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
         if constexpr (kBg) {  // incoherent background: one more component of the model intensity
             const int pix = id + k1 * RN;
             ic += __ldg(a.bg + pix);
-            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
+            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io[k1], ic));
         }
         float f;
         if (mode == COL_PROJECT) {
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
         if (bgp) {
             const int pix = id + k1 * RN;
             ic += __ldg(bgp + pix);
-            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : fmaxf(io, 0.f) / fmaxf(ic, 1e-30f));
+            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
         }
         if (mode == COL_PROJECT) {
             float ratio;
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, SplitShape<N>::ColBlocks) k_row_proj
         const bool masked = a.mask[pix] != 0;
         if (bgp) {  // incoherent background in the detector plane
             ic += __ldg(bgp + pix);
-            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, fmaxf(io[k1], 0.f) / fmaxf(ic, 1e-30f));
+            if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, quotient(io[k1], ic));
         }
         if (!masked) llk += llk_term_fast(ic, io[k1]);
         const float f = masked ? 0.f : amp_ratio(io[k1], ic) - 1.0f;
