@@ -16,10 +16,12 @@
 // frames in a cluster of 8 or 16 blocks, the transpose through distributed shared
 // memory, took 354 - 450 us: that exchange sustains 3.2 - 4.2 TB/s.
 #pragma once
-#include "kernels_reg.cuh"
+#include "kernels_split.cuh"
 
 namespace ptx {
 
+template <int N>
+constexpr bool fft_split() { return use_split<N>() && Plan<N>::M > Plan<N>::R; }
 template <int N>
 constexpr bool fft_whole() { return Plan<N>::M > 1 && RegShape<N>::L == N; }
 
@@ -118,6 +120,106 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_fft_cols_r
             for (int k1 = 0; k1 < M; ++k1) st_hint(base + (size_t)(k2 + R * k1) * N + c, cscale(u[k1], invN), ef);
         }
     }
+}
+
+// The same with the column transform split between the passes (kernels_split.cuh),
+// where the second factor is the larger one: the column pass then has no idle
+// threads in its first factor and no transpose.  200 frames of 512^2 288 -> 260 us,
+// 300 of 400^2 315 -> 278, 400 of 384^2 356 -> 313; at 256^2 305 against 309 for 1024
+// frames but 16.5 against 14.7 for 40, so it keeps the passes above.  Rows n1 + M l of a frame: row transforms, then the
+// first factor of the columns, back into the same rows (value k2 in row n1 + M k2).
+// grid (M, frames)
+template <int N, int DIR>
+__global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_fft_rows_s(float2* data) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, P = S::P;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;
+    float2* buf = sm + N;
+    pdl_launch_dependents();
+    load_twiddles<N>(tw);
+    const int n1b = blockIdx.x;
+    float2* base = data + (size_t)blockIdx.y * N * N;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < S::I1; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < R * M) {
+            const int line = w / M, n1 = w - line * M;
+            const float2* src = base + (size_t)(n1b + M * line) * N + n1;
+            const uint64_t ef = policy_evict_first();
+            float2 v[R];
+#pragma unroll
+            for (int n2 = 0; n2 < R; ++n2) v[n2] = ld_hint(src + M * n2, ef);
+            Dft<R, DIR>::run(v);
+            float2* o = buf + line * P + n1;
+            o[0] = v[0];
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, DIR>(tw, k2, n1));
+        }
+    }
+    split_row_sync<N>();
+    float2 u[S::I2][M];
+#pragma unroll
+    for (int i = 0; i < S::I2; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < R * R) {
+            const int line = w / R, k2 = w - line * R;
+            const float2* src = buf + line * P + k2 * (M + 1);
+#pragma unroll
+            for (int n1 = 0; n1 < M; ++n1) u[i][n1] = src[n1];
+            Dft<M, DIR>::run(u[i]);
+        }
+    }
+    split_row_sync<N>();
+#pragma unroll
+    for (int i = 0; i < S::I2; ++i) {
+        const int w = threadIdx.x + i * kThreads;
+        if (w < R * R) {
+            const int line = w / R, k2 = w - line * R;
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) buf[line * P + k2 + R * k1] = u[i][k1];
+        }
+    }
+    __syncthreads();
+    pdl_wait();
+#pragma unroll
+    for (int i = 0; i < S::I1; ++i) {
+        const int kx = threadIdx.x + i * kThreads;
+        if (kx < N) {
+            float2 v[R];
+#pragma unroll
+            for (int l = 0; l < R; ++l) v[l] = buf[l * P + kx];
+            Dft<R, DIR>::run(v);
+            const uint64_t el = policy_evict_last();
+            st_hint(base + (size_t)n1b * N + kx, v[0], el);
+#pragma unroll
+            for (int k2 = 1; k2 < R; ++k2)
+                st_hint(base + (size_t)(n1b + M * k2) * N + kx, cmul(v[k2], tw_get<N, DIR>(tw, k2, n1b)), el);
+        }
+    }
+}
+
+// Columns [x C, x C + C) of a frame: thread (k2, c) finds its M values in rows
+// n1 + M k2 and leaves the results in rows k2 + R k1, so the block, which owns its
+// columns, reads all of them before it writes.  grid (N / C, frames)
+template <int N, int DIR>
+__global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks) k_fft_cols_s(float2* data) {
+    using S = SplitShape<N>;
+    constexpr int R = S::R, M = S::M, C = reg_cols<N>();
+    pdl_launch_dependents();
+    const int k2 = threadIdx.x / C, c = threadIdx.x - k2 * C;
+    float2* base = data + (size_t)blockIdx.y * N * N + (size_t)blockIdx.x * C + c;
+    pdl_wait();
+    const uint64_t ef = policy_evict_first();
+    float2 u[M];
+#pragma unroll
+    for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(base + (size_t)(n1 + M * k2) * N, ef);
+    Dft<M, DIR>::run(u);
+    __syncthreads();
+    constexpr float invN = 1.0f / float(N);
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) st_hint(base + (size_t)(k2 + R * k1) * N, cscale(u[k1], invN), ef);
 }
 
 // grid (frames): one whole frame per block
@@ -228,8 +330,13 @@ void launch_fft2_r(float2* data, int nframes, cudaStream_t s) {
             const int n = nframes - f < chunk ? nframes - f : chunk;
             float2* d = data + (size_t)f * N * N;
             // the first launch of the call follows whatever the stream holds: plain
-            launch_dep(k_fft_rows_r<N, DIR>, dim3(N / S::L, n), sizeof(float2) * (N + (size_t)S::L * S::P), s, f > 0, d);
-            launch_dep(k_fft_cols_r<N, DIR>, dim3(N / S::C, n), sizeof(float2) * (N + (size_t)S::C * S::P), s, true, d);
+            if constexpr (fft_split<N>()) {
+                launch_dep(k_fft_rows_s<N, DIR>, dim3(Plan<N>::M, n), smem_row_fwd_s<N>(), s, f > 0, d);
+                launch_dep(k_fft_cols_s<N, DIR>, dim3(N / S::C, n), 0, s, true, d);
+            } else {
+                launch_dep(k_fft_rows_r<N, DIR>, dim3(N / S::L, n), sizeof(float2) * (N + (size_t)S::L * S::P), s, f > 0, d);
+                launch_dep(k_fft_cols_r<N, DIR>, dim3(N / S::C, n), sizeof(float2) * (N + (size_t)S::C * S::P), s, true, d);
+            }
         }
     }
 }
@@ -247,6 +354,9 @@ cudaError_t set_attrs_fft() {
     if constexpr (fft_whole<N>()) {
         if ((e = fft_attrs<N>(k_fft_frame_r<N, -1>))) return e;
         return fft_attrs<N>(k_fft_frame_r<N, +1>);
+    } else if constexpr (fft_split<N>()) {
+        if ((e = fft_attrs<N>(k_fft_rows_s<N, -1>))) return e;
+        return fft_attrs<N>(k_fft_rows_s<N, +1>);
     } else {
         if ((e = fft_attrs<N>(k_fft_rows_r<N, -1>))) return e;
         if ((e = fft_attrs<N>(k_fft_rows_r<N, +1>))) return e;
