@@ -359,7 +359,7 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     if (per_sm <= 0) per_sm = 2;
     int resident = per_sm * sm_count();
     int rowblk = p.N / h.L3 * p.K;
-    if (h.ks->col_s && h.ks->M > h.ks->R) {  // k_row_bwd_s2: two blocks per SM, M of them per frame and mode
+    if (h.ks->row_bwd_s) {  // two blocks per SM, M of them per frame and mode
         resident = 2 * sm_count();
         rowblk = h.ks->M * p.K;
     }
@@ -368,7 +368,7 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     // (DM cycle, 4000 x 256^2, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us; 300
     // frames 270 with 19 and 14, 273 with 10; 150 x 512^2, 9 / 6 / 4: 631 / 620 / 625; 203 x 400^2, 12 / 8 / 6:
     // 644 / 638 / 642)
-    if (slots == 0 && lanes > 1 && h.ks->col_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
+    if (slots == 0 && lanes > 1 && h.ks->row_bwd_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
     // (several modes of large frames: one slot would leave a third of the SMs with half their blocks;
     // 300 three-mode 512^2 frames, 1 / 2 / 3 slots: 3966 / 3877 / 3893 us)
     if (slots == 0 && G == 1 && 2 * resident >= 3 * rowblk) G = 2;
@@ -438,7 +438,7 @@ size_t layout_problem(ProbHost& h) {
     h.lay.mbits = o;
     if (use_reg_kernels(h.ks, p.K)) o = align_up(o + sizeof(uint32_t) * (size_t)(p.N / h.ks->reg_cols) * kThreads);
     h.lay.mbits_s = o;
-    if (h.ks->col_s) o = align_up(o + sizeof(uint32_t) * (size_t)h.ks->R * p.N);
+    if (h.ks->split_ls) o = align_up(o + sizeof(uint32_t) * (size_t)h.ks->R * p.N);
     h.lay.nf_t = o;
     if (p.nearfield > 0.0) o = align_up(o + sizeof(float2) * (size_t)p.N);
     h.lay.bg_acc = o;
@@ -693,7 +693,7 @@ void fill_args(ptx_handle* h, ProbHost& ph) {
     a.ls_part = (double*)(h->scratch + ph.lay.ls_part);
     a.err_flag = h->err_dev;
     a.mbits = (const uint32_t*)(h->scratch + ph.lay.mbits);
-    a.mbits_s = ph.ks->col_s ? (const uint32_t*)(h->scratch + ph.lay.mbits_s) : nullptr;
+    a.mbits_s = ph.ks->split_ls ? (const uint32_t*)(h->scratch + ph.lay.mbits_s) : nullptr;
     a.nf_t = ph.p.nearfield > 0.0 ? (const float2*)(h->scratch + ph.lay.nf_t) : nullptr;
     a.bg = ph.p.background;
     a.bg_acc = nullptr;  // set only for the column passes of AP cycles that update the background
@@ -1306,7 +1306,7 @@ ptx_status ptx_create(ptx_handle** out, const ptx_problem* probs, int32_t nprob,
                                     cudaMemcpyHostToDevice, s);
                 if (e != cudaSuccess) break;
             }
-            if (ph.ks->col_s) {
+            if (ph.ks->split_ls) {
                 mbits_s_host[i] = mask_bits_split(ph.ks, ph.p.N, ph.p.mask);
                 e = cudaMemcpyAsync(h->scratch + ph.lay.mbits_s, mbits_s_host[i].data(),
                                     sizeof(uint32_t) * mbits_s_host[i].size(), cudaMemcpyHostToDevice, s);

@@ -27,9 +27,16 @@
 
 namespace ptx {
 
+// Sizes whose LLK, cycles and gradient take the split passes.  At 128^2 half the
+// threads of a row block idle in the 16-point factors (2500-frame LLK 228 -> 265 us);
+// its line search gains all the same (CG step of 900 frames 424 -> 389 us).
 template <int N>
 __host__ __device__ constexpr bool use_split() {
-    return N == 256 || N >= 384;
+    return N >= 160;
+}
+template <int N>
+__host__ __device__ constexpr bool use_split_ls() {
+    return N >= 128;
 }
 // sizes whose near-field passes are split too (the row pass at the detector keeps rows in a warp)
 template <int N>
@@ -399,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_row_fwd_
 // Line search, column pass (k_col_ls_r's sums): second factors of every wave of
 // the thread's pixels.  grid (N / C, frames in batch)
 template <int N, bool kModes, bool kThree>
-__global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, kThree>() * kThreads / SplitShape<N>::TC))
+__global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, kThree>() * kThreads + SplitShape<N>::TC - 1) / SplitShape<N>::TC)
     k_col_ls_s(ProbArgs a, int j0) {
     using S = SplitShape<N>;
     constexpr int R = S::R, M = S::M, RN = R * N, kWaves = kThree ? 3 : 2;
@@ -486,6 +493,9 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, k
 // Backward: first factor of the inverse column transform, row transforms, then
 // Psi' and the probe sums (or the gradient) as in the backward row pass of
 // kernels_reg.cuh.  grid (M, G K); blockIdx.y = slot * K + mode
+// The object rows are staged by the thread (M < R) or the warp that uses them.
+// DM cycle / gradient of 900 frames, kernels_reg.cuh -> split passes: 160^2 391 -> 373 /
+// 300 -> 276 us, 192^2 520 -> 496 / 413 -> 368, 224^2 711 -> 698 / 579 -> 525.
 template <int N, int kForm>
 __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, int nb, int mode_arg, int upd_obj_arg,
                                                            int upd_probe_arg) {
@@ -494,42 +504,49 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, i
     const int upd_obj = kForm >= 2 ? 1 : upd_obj_arg;
     using S = SplitShape<N>;
     constexpr int R = S::R, M = S::M, P = S::P;
-    static_assert(S::kWarpRows && S::I2 == 1 && S::I1 == 1, "one item per thread, rows within a warp");
+    constexpr bool kWarp = S::kWarpRows;
+    static_assert(R * R == kThreads && M <= R && N <= kThreads, "one item per thread");
     extern __shared__ __align__(16) float2 sm[];
     float2* tw = sm;
-    float2* stage = sm + N;         // [R][N] next frame's values (cp.async)
-    float2* ostage = stage + R * N; // [R][N] next frame's object rows (cp.async)
-    float2* buf = ostage + R * N;
+    float2* stage = sm + N;          // [R][N] next frame's values (cp.async)
+    float2* ostage = stage + R * N;  // next frame's object values: [R][N], or [M][thread] (cp.async)
+    float2* buf = ostage + M * kThreads;
     load_twiddles<N>(tw);
-    const int K = a.K, n1b = blockIdx.x;
+    const int K = a.K, n1b = blockIdx.x, t = threadIdx.x;
     const int slot = blockIdx.y / K, k = blockIdx.y - slot * K;
     const int G = gridDim.y / K;
     const bool acc_p = upd_probe != 0, acc_o = upd_obj != 0;
     const bool stage_obj = mode != BWD_GRAD || acc_p;
-    const int line = threadIdx.x / R, k2t = threadIdx.x - line * R;  // R == M: the same row in both factors
+    const int line = t / R, k2t = t - line * R;  // second factor: pixels k2t + R k1 of row `line`
+    const int l1 = t / M, n1 = t - l1 * M;       // first factor (t < R M): row l1, elements n1 + M i
     const int y = n1b + M * line;
     auto prefetch_spec = [&](int b) {
         const float2* src = a.spec + (((size_t)b * K + k) * M + n1b) * R * N;
         const uint64_t ef = policy_evict_first();  // the stack's last read
 #pragma unroll
-        for (int i = 0; i < R * N / 2 / kThreads; ++i) {
-            const int e = 2 * (threadIdx.x + i * kThreads);
-            cp_async16_hint(stage + e, src + e, ef);
+        for (int i = 0; i < (R * N / 2 + kThreads - 1) / kThreads; ++i) {
+            const int e = 2 * (t + i * kThreads);
+            if (R * N / 2 % kThreads == 0 || e < R * N) cp_async16_hint(stage + e, src + e, ef);
         }
         cp_async_commit();
     };
-    // the object rows of this warp's lines (8-byte aligned only)
     auto prefetch_obj = [&](int b) {
         if (stage_obj) {
             const int2 q = a.pos[j0 + b];
-            constexpr int kLines = 32 / R;
+            if constexpr (kWarp) {  // the rows of this warp's lines (8-byte aligned only)
+                constexpr int kLines = 32 / R;
 #pragma unroll
-            for (int l = 0; l < kLines; ++l) {
-                const int row = (threadIdx.x >> 5) * kLines + l;
-                const float2* src = a.obj + (size_t)(q.x + n1b + M * row) * a.Wo + q.y + (threadIdx.x & 31);
-                float2* dst = ostage + row * N + (threadIdx.x & 31);
+                for (int l = 0; l < kLines; ++l) {
+                    const int row = (t >> 5) * kLines + l;
+                    const float2* src = a.obj + (size_t)(q.x + n1b + M * row) * a.Wo + q.y + (t & 31);
+                    float2* dst = ostage + row * N + (t & 31);
 #pragma unroll
-                for (int i = 0; i < N / 32; ++i) cp_async8(dst + 32 * i, src + 32 * i);
+                    for (int i = 0; i < N / 32; ++i) cp_async8(dst + 32 * i, src + 32 * i);
+                }
+            } else {
+                const float2* src = a.obj + (size_t)(q.x + y) * a.Wo + q.y + k2t;
+#pragma unroll
+                for (int k1 = 0; k1 < M; ++k1) cp_async8(ostage + k1 * kThreads + t, src + R * k1);
             }
         }
         cp_async_commit();
@@ -551,61 +568,64 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, i
         const int2 p = a.pos[j];
         cp_async_wait_all();
         __syncthreads();
-        {  // columns: thread kx, first factor of the inverse over k2 -> rows n1b + M l
-            const int kx = threadIdx.x;
+        if (N == kThreads || t < N) {  // columns: thread kx, first factor of the inverse over k2 -> rows n1b + M l
             float2 v[R];
-            v[0] = stage[kx];
+            v[0] = stage[t];
 #pragma unroll
-            for (int k2 = 1; k2 < R; ++k2) v[k2] = cmul(stage[k2 * N + kx], tw_get<N, +1>(tw, k2, n1b));
+            for (int k2 = 1; k2 < R; ++k2) v[k2] = cmul(stage[k2 * N + t], tw_get<N, +1>(tw, k2, n1b));
             Dft<R, +1>::run(v);
 #pragma unroll
-            for (int l = 0; l < R; ++l) buf[l * P + kx] = v[l];
+            for (int l = 0; l < R; ++l) buf[l * P + t] = v[l];
         }
         __syncthreads();
         if (b + G < nb) prefetch_spec(b + G);  // the stage is free again
         {
-            const float2* src = buf + line * P + k2t;
             float2 v[R];
+            const bool on = kWarp || t < R * M;
+            if (on) {
 #pragma unroll
-            for (int n2 = 0; n2 < R; ++n2) v[n2] = src[M * n2];
-            __syncwarp();
-            Dft<R, +1>::run(v);
-            float2* o = buf + line * P + k2t;
-            o[0] = v[0];
+                for (int n2 = 0; n2 < R; ++n2) v[n2] = buf[l1 * P + n1 + M * n2];
+            }
+            split_row_sync<N>();
+            if (on) {
+                Dft<R, +1>::run(v);
+                float2* o = buf + l1 * P + n1;
+                o[0] = v[0];
 #pragma unroll
-            for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, +1>(tw, k2, k2t));
+                for (int k2 = 1; k2 < R; ++k2) o[k2 * (M + 1)] = cmul(v[k2], tw_get<N, +1>(tw, k2, n1));
+            }
         }
-        __syncwarp();
+        split_row_sync<N>();
         float2 u[M];
 #pragma unroll
-        for (int n1 = 0; n1 < M; ++n1) u[n1] = buf[line * P + k2t * (M + 1) + n1];
+        for (int i = 0; i < M; ++i) u[i] = buf[line * P + k2t * (M + 1) + i];
         Dft<M, +1>::run(u);
         const size_t orow = (size_t)(p.x + y) * a.Wo + p.y + k2t;
-        const float2* ob = stage_obj ? ostage + line * N + k2t : a.obj + orow;
         float2* ps = (mode != BWD_GRAD) ? a.psi + (((size_t)j * K + k) * N + y) * N + k2t : nullptr;
 #pragma unroll
         for (int k1 = 0; k1 < M; ++k1) {
-            const float2 obv = ob[R * k1];
+            const float2 obv = !stage_obj ? make_float2(0.f, 0.f)
+                                          : (kWarp ? ostage[line * N + k2t + R * k1] : ostage[k1 * kThreads + t]);
             float2 wv;
             if (mode == BWD_GRAD) {
                 wv = u[k1];
                 if (acc_o) {
-                    const float2 t = cconjmul(pr_r[k1], wv);
-                    red_add_v2(a.grad_obj + orow + R * k1, t.x, t.y);
+                    const float2 c = cconjmul(pr_r[k1], wv);
+                    red_add_v2(a.grad_obj + orow + R * k1, c.x, c.y);
                 }
             } else {
                 wv = cadd(cmul(pr_r[k1], obv), u[k1]);
                 __stcs(ps + R * k1, wv);
             }
             if (acc_p) {
-                const float2 t = cconjmul(obv, wv);
-                np_r[k1].x += t.x;
-                np_r[k1].y += t.y;
+                const float2 c = cconjmul(obv, wv);
+                np_r[k1].x += c.x;
+                np_r[k1].y += c.y;
                 dp_r[k1] += cnorm(obv);
             }
         }
-        __syncwarp();
-        if (b + G < nb) prefetch_obj(b + G);  // this warp's object rows are free again
+        if constexpr (kWarp) __syncwarp();
+        if (b + G < nb) prefetch_obj(b + G);  // the object values are free again
     }
     if (acc_p) {
         const size_t pidx = ((size_t)k * N + y) * N + k2t;
@@ -841,8 +861,8 @@ template <int N>
 size_t smem_row_fwd_s() { return sizeof(float2) * (N + (size_t)Plan<N>::R * reg_pitch<N>()); }
 template <int N>
 size_t smem_row_bwd_s() {
-    constexpr size_t stages = Plan<N>::M > Plan<N>::R ? 0 : 2 * N;
-    return sizeof(float2) * (N + Plan<N>::R * (stages + reg_pitch<N>()));
+    constexpr size_t stages = Plan<N>::M > Plan<N>::R ? 0 : Plan<N>::R * N + Plan<N>::M * kThreads;
+    return sizeof(float2) * (N + stages + Plan<N>::R * reg_pitch<N>());
 }
 
 template <int N>
@@ -856,8 +876,7 @@ void launch_col_s(const ProbArgs& a, int j0, int nb, int mode, cudaStream_t s, b
     auto k = a.K > 1 ? (mode == COL_PROJECT && !a.bg ? k_col_modes_s<N, true> : k_col_modes_s<N, false>)
              : a.bg  ? (mode == COL_PROJECT ? k_col_s<N, true, true> : k_col_s<N, true, false>)
                      : (mode == COL_PROJECT ? k_col_s<N, false, true> : k_col_s<N, false, false>);
-    static_assert(SplitShape<N>::TC == kThreads, "launch_dep's block size");
-    launch_dep(k, grid, 0, s, pdl, a, j0, mode);
+    launch_dep<SplitShape<N>::TC>(k, grid, 0, s, pdl, a, j0, mode);
 }
 // The cycle's form (Psi' and probe sums), the gradient of the object and of both
 // parts have instantiations of their own (kForm 1, 2, 3), the rest takes its flags
@@ -883,7 +902,7 @@ void launch_row_bwd_s(const ProbArgs& a, int j0, int nb, int G, int mode, int up
 // Near field (pdl: as for the passes above) and line search.
 template <int N>
 void launch_col_nf_s(const ProbArgs& a, int nb, int dir, cudaStream_t s, bool pdl) {
-    launch_dep(dir < 0 ? k_col_nf_s<N, -1> : k_col_nf_s<N, +1>, dim3(N / reg_cols<N>(), nb), 0, s, pdl, a);
+    launch_dep<SplitShape<N>::TC>(dir < 0 ? k_col_nf_s<N, -1> : k_col_nf_s<N, +1>, dim3(N / reg_cols<N>(), nb), 0, s, pdl, a);
 }
 template <int N>
 void launch_row_proj_s(const ProbArgs& a, int j0, int nb, int llk_only, cudaStream_t s, bool pdl) {
@@ -900,7 +919,7 @@ void launch_col_ls_s(const ProbArgs& a, int j0, int nb, int pdl, cudaStream_t s)
     const bool three = ls_waves(a.dir_obj, a.dir_probe) == 3;
     auto k = a.K == 1 ? (three ? k_col_ls_s<N, false, true> : k_col_ls_s<N, false, false>)
                       : (three ? k_col_ls_s<N, true, true> : k_col_ls_s<N, true, false>);
-    launch_dep(k, dim3(N / reg_cols<N>(), nb), 0, s, pdl != 0, a, j0);
+    launch_dep<SplitShape<N>::TC>(k, dim3(N / reg_cols<N>(), nb), 0, s, pdl != 0, a, j0);
 }
 
 template <class F>
@@ -912,11 +931,12 @@ cudaError_t split_attrs(F f) {
 }
 template <int N>
 cudaError_t set_attrs_split() {
+    cudaError_t e;
+    if constexpr (use_split_ls<N>())
+        if ((e = split_attrs(k_row_fwd_ls_s<N>))) return e;
     if constexpr (use_split<N>()) {
-        cudaError_t e;
         if ((e = split_attrs(k_row_fwd_s<N, false>))) return e;
         if ((e = split_attrs(k_row_fwd_s<N, true>))) return e;
-        if ((e = split_attrs(k_row_fwd_ls_s<N>))) return e;
         if constexpr (use_split_nf<N>()) {
             if ((e = split_attrs(k_row_proj_s<N, false>))) return e;
             if ((e = split_attrs(k_row_proj_s<N, true>))) return e;

@@ -187,7 +187,9 @@ def _scan(N, K, J, masked, seed):
 
 # one frame; fewer and more frames than the backward pass has slots; several modes; parts of the update left out
 @pytest.mark.parametrize("N,K,J,masked,upd_o,upd_p", [
-    (256, 1, 1, True, True, True), (256, 1, 3, False, False, True), (256, 1, 23, True, True, False),
+    (160, 1, 40, True, True, True), (160, 2, 3, False, True, False), (192, 1, 1, True, True, True),
+    (192, 3, 2, True, False, True), (224, 1, 31, False, True, True), (256, 1, 1, True, True, True),
+    (256, 1, 3, False, False, True), (256, 1, 23, True, True, False),
     (256, 2, 2, True, True, True), (256, 3, 9, False, False, False), (384, 1, 1, False, True, True),
     (384, 2, 7, True, True, False), (400, 1, 26, True, True, True), (400, 3, 2, False, False, True),
     (448, 1, 5, True, True, True), (512, 1, 18, False, True, True), (512, 3, 2, True, True, True),
@@ -207,7 +209,8 @@ def test_split_passes_dm_cycle(N, K, J, masked, upd_o, upd_p):
     pb.close()
 
 
-@pytest.mark.parametrize("N,K,J,masked", [(256, 1, 1, False), (256, 1, 21, True), (256, 3, 4, True), (384, 1, 3, True),
+@pytest.mark.parametrize("N,K,J,masked", [(160, 1, 33, True), (192, 2, 3, False), (224, 1, 1, True),
+                                          (256, 1, 1, False), (256, 1, 21, True), (256, 3, 4, True), (384, 1, 3, True),
                                           (400, 2, 9, False), (448, 1, 2, True), (512, 1, 11, True), (512, 3, 2, False)])
 @pytest.mark.parametrize("parts", ["obj", "probe", "both"])
 def test_split_passes_gradient(N, K, J, masked, parts):
