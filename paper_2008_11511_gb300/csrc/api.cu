@@ -322,22 +322,29 @@ ptx_status check_problem(const ptx_problem& p, int idx) {
     return PTX_OK;
 }
 
-// Frames per batch when at most `most` fit: J frames in as few batches as that
-// allows (a multiple of the lanes when there are several), all of about the same
-// size, because a short last batch costs nearly a full one.  With one lane nothing
-// fills the last wave of a launch but the head of the next one, so `most` is cut
-// to whole waves of the column pass (`wave` frames each, the pass with the fewest
-// resident blocks): 1000 x 256^2 gradient, 64 -> 125 -> 112 frames per batch,
-// 831 -> 765 -> 755 us; 2500 x 128^2 LLK, 256 -> 500 -> 417 frames, 262 -> 249 ->
-// 244 us; two CG steps on 1000 x 256^2, line search in 62 -> 56 frames, 3.68 ->
-// 3.61 ms.  With two lanes, each filling the other's tails, 48 to 64 frames are
-// within 1 % (4000 x 256^2 DM cycle) and whole waves (38 frames) 2 % slower.
+// Frames per batch when at most `most` fit.  With one lane: J frames in as few
+// batches as that allows, all of about the same size, because a short last batch
+// costs nearly a full one, and `most` is cut to whole waves of the column pass
+// (`wave` frames each, the pass with the fewest resident blocks), because nothing
+// fills the last wave of a launch but the head of the next one: 1000 x 256^2
+// gradient, 64 -> 125 -> 112 frames per batch, 831 -> 765 -> 755 us; 2500 x 128^2
+// LLK, 256 -> 500 -> 417 frames, 262 -> 249 -> 244 us; two CG steps on 1000 x 256^2,
+// line search in 62 -> 56 frames, 3.68 -> 3.61 ms.  Several lanes fill each other's
+// tails (4000 x 256^2 DM cycle: 48 to 64 frames are within 1 %, whole waves of 38
+// frames 2 % slower), so there it is `most` frames, then the rest, unless a few
+// batches would leave a lane idle at the end: 30 x 400^2 in 13 + 13 + 4 frames 376 us,
+// in 4 x 8 333; 107 x 512^2 in 6 x 16 + 11 497, in 8 x 14 468.
 size_t even_batch(size_t most, size_t J, int lanes, double wave) {
     most = std::max<size_t>(1, std::min<size_t>(most, 32768));  // grid.y limit of the batch kernels
-    if (lanes == 1 && wave >= 1.0 && most < J && (double)most > wave)
-        most = (size_t)(std::floor((double)most / wave) * wave);
-    size_t n = (J + most - 1) / most;
-    if (n > 1) n = (n + lanes - 1) / lanes * lanes;
+    if (most >= J) return J;
+    if (lanes > 1) {
+        size_t n = (J + most - 1) / most;
+        if (n > 16 || (n % lanes == 0 && 4 * (J - (n - 1) * most) >= 3 * most)) return most;
+        n = (n + lanes - 1) / lanes * lanes;
+        return (J + n - 1) / n;
+    }
+    if (wave >= 1.0 && (double)most > wave) most = (size_t)(std::floor((double)most / wave) * wave);
+    const size_t n = (J + most - 1) / most;
     return (J + n - 1) / n;
 }
 double frames_per_wave(int per_sm, int blocks_per_frame) { return (double)per_sm * sm_count() / blocks_per_frame; }
@@ -357,21 +364,14 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     // frames and flushes its probe sums once)
     int per_sm = h.ks->row_bwd_per_sm();
     if (per_sm <= 0) per_sm = 2;
-    int resident = per_sm * sm_count();
-    int rowblk = p.N / h.L3 * p.K;
-    if (h.ks->row_bwd_s) {  // two blocks per SM, M of them per frame and mode
-        resident = 2 * sm_count();
-        rowblk = h.ks->M * p.K;
-    }
+    const int resident = per_sm * sm_count();
+    const int rowblk = p.N / h.L3 * p.K;
     int G = slots > 0 ? slots : resident / rowblk;
-    // split passes in several lanes: two thirds of that, leaving SMs to the other lanes' passes
-    // (DM cycle, 4000 x 256^2, 19 / 16 / 14 / 12 / 10 / 8 slots: 3193 / 3145 / 3135 / 3121 / 3112 / 3146 us; 300
-    // frames 270 with 19 and 14, 273 with 10; 150 x 512^2, 9 / 6 / 4: 631 / 620 / 625; 203 x 400^2, 12 / 8 / 6:
-    // 644 / 638 / 642)
-    if (slots == 0 && lanes > 1 && h.ks->row_bwd_s && p.K == 1) G = (2 * resident / rowblk + 1) / 3;
-    // (several modes of large frames: one slot would leave a third of the SMs with half their blocks;
-    // 300 three-mode 512^2 frames, 1 / 2 / 3 slots: 3966 / 3877 / 3893 us)
-    if (slots == 0 && G == 1 && 2 * resident >= 3 * rowblk) G = 2;
+    // (DM cycles: 150 x 512^2, 4 / 6 / 9 slots 625 / 620 / 631 us, 203 x 400^2, 6 / 8 / 12: 642 / 638 / 644; 4000 x
+    // 256^2, 19 / 16 / 12: 3193 / 3145 / 3121, which would regroup the probe's sums for 2 %)
+    // the split passes of several modes above 256^2 have half the row blocks: 300 three-mode 512^2 frames, 1 / 2 / 3
+    // slots: 4152 / 3710 / 3647 us
+    if (slots == 0 && p.K > 1 && h.ks->col_s && h.ks->M > h.ks->R) G = 2 * sm_count() / (h.ks->M * p.K);
     if (G > h.B) G = h.B;
     if (G < 1) G = 1;
     h.G3 = G;
