@@ -17,7 +17,7 @@
 // -> 13.9 us (from two transposes and three barriers to none: 64 % issue active, the
 // projection's arithmetic now half of it), forward row pass 20.8 -> 21.3, backward
 // 20.7 -> 22.6 with the column factor added, near-field column pass 19.1 -> 10.7,
-// line-search column pass 49 -> 27.  In the cycle: 4000 frames, DM 3.41 -> 3.13 ms; near field,
+// line-search column pass 49 -> 27.  In the cycle: 4000 frames, DM 3.41 -> 3.22 ms; near field,
 // 500 frames, 716 -> 630 us; gradient of 1000 frames 755 -> 685 us; two CG steps
 // 3.60 -> 2.85 ms; three-mode CG step of 150 frames 944 -> 854 us.  The passes of
 // kernels_reg.cuh keep the other sizes and, at 256^2, the stack order that the
