@@ -224,7 +224,7 @@ ptx_status ptx_accumulators(ptx_handle* h, int32_t p, void** obj_acc, size_t* ob
 /* Set a scalar parameter: "alpha_obj" or "alpha_probe" (inertia factors of the
  * normalisation, default 0.01 each, must be >= 0); "lanes" (batches in flight per
  * cycle, 1..4, default 2); "batch_frames" (upper bound on frames per batch, 0 =
- * as many as the work stack holds); "bwd_slots" (frame slots of the row-backward
+ * as many as the work stack holds; a few batches are evened out below it); "bwd_slots" (frame slots of the row-backward
  * pass: blocks per row band, each looping over every bwd_slots-th frame of a
  * batch and flushing its probe sums once; 0, default: as many as are resident
  * at once); "persistent" (0, default; 1: the batch passes of every problem of
@@ -242,11 +242,11 @@ ptx_status ptx_accumulators(ptx_handle* h, int32_t p, void** obj_acc, size_t* ob
  * default; 1: with a tensor-core form, the forward and backward row passes of
  * problems with N = 256 and one mode, or N = 512 and any number of modes, run
  * their DFT stages on the tensor cores too, so that every DFT stage of the
- * cycle is in that form); "pdl" (1, default: the FP32 register passes of
- * far-field problems without a background (forward row, column and backward
- * row passes of the one-mode AP / DM cycle within each lane, of ptx_llk,
- * ptx_ml_grad and the ML cycles' gradients; the one-mode line-search passes)
- * are launched as
+ * cycle is in that form); "pdl" (1, default: the FP32 register passes
+ * (forward row, column and backward row passes of the one-mode AP / DM cycle
+ * within each lane, of ptx_llk, ptx_ml_grad and the ML cycles' gradients; the
+ * line-search passes; far field with or without a background, and the near field
+ * at N = 256) are launched as
  * programmatic dependents of the pass before them, so that a pass's first
  * blocks load their inputs while the previous pass's last blocks finish; 0:
  * plain launches, each pass after the whole previous one); "tma" (0, default:
