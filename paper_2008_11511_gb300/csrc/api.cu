@@ -332,14 +332,16 @@ ptx_status check_problem(const ptx_problem& p, int idx) {
 // line search in 62 -> 56 frames, 3.68 -> 3.61 ms.  Several lanes fill each other's
 // tails (4000 x 256^2 DM cycle: 48 to 64 frames are within 1 %, whole waves of 38
 // frames 2 % slower), so there it is `most` frames, then the rest, unless a few
-// batches would leave a lane idle at the end: 30 x 400^2 in 13 + 13 + 4 frames 376 us,
+// batches of few frames would leave a lane idle at the end (with many frames to a
+// batch little is lost, and evening them would regroup the probe's sums): 30 x 400^2 in 13 + 13 + 4 frames 376 us,
 // in 4 x 8 333; 107 x 512^2 in 6 x 16 + 11 497, in 8 x 14 468.
+constexpr size_t kFewFrames = 32;
 size_t even_batch(size_t most, size_t J, int lanes, double wave) {
     most = std::max<size_t>(1, std::min<size_t>(most, 32768));  // grid.y limit of the batch kernels
     if (most >= J) return J;
     if (lanes > 1) {
         size_t n = (J + most - 1) / most;
-        if (n > 16 || (n % lanes == 0 && 4 * (J - (n - 1) * most) >= 3 * most)) return most;
+        if (n > 16 || most > kFewFrames || (n % lanes == 0 && 4 * (J - (n - 1) * most) >= 3 * most)) return most;
         n = (n + lanes - 1) / lanes * lanes;
         return (J + n - 1) / n;
     }
@@ -1020,7 +1022,10 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
         const bool pdl = pass_pdl(h, ph) && !tc_col && ph.p.K == 1;
         const bool tma_col = h->tma && ph.tma_io && ks->col_tma && ph.p.nearfield <= 0.0 && !ph.p.background;
         const bool split = split_passes(ph) && !tc_col && !tma_col;
-        const bool whole = frame_launch(h, ph);
+        // (every frame at once: with more, a block's probe sums would run over frames of several batches, and the
+        // rounding of sums grouped otherwise grows from cycle to cycle near the waves' zeros: 2453 frames of 64^2,
+        // three DM cycles, Psi off by 2.7e-5 of its norm for 8 % of the time)
+        const bool whole = frame_launch(h, ph) && ph.p.J <= frame_blocks(ph.p.N);
         if (whole) {
             const int lane = next_lane;
             next_lane = (next_lane + 1) % lanes;

@@ -391,12 +391,6 @@ __global__ void k_set_ctl(Ctl* ctl, double* llk_out, int nprob) {
 
 namespace ptx {
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // A float as a double by its bits: the conversion instruction shares the FP64
 // pipe (a few lanes per clock) with the products it feeds.  Exact for zero and
 // normal values; others take the instruction.

@@ -9,9 +9,10 @@
 // transpose is in place (a column's second factor rewrites exactly the rows it
 // read) or within a warp, and a block loops over its frames with its pixels'
 // probe sums in registers, flushing them once.  Two blocks of 512 threads per
-// SM at 64^2 (some of the sums spill) beat one without spills: 6000 frames, DM
-// cycle 609 (three passes) -> 582 us (one block per SM: 625), LLK 163 -> 131 (163).
-// 100 frames of 64^2, five AP cycles: 180 -> 170 us.
+// SM at 64^2 (some of the sums spill) beat one without spills: LLK of 6000 frames
+// 163 (three passes) -> 131 us (one block per SM: 163), DM cycle 609 -> 582 (625).
+// The cycles take it while every frame has a block of its own: 100 frames of 64^2,
+// five AP cycles, 180 -> 170 us.
 #pragma once
 #include "kernels_reg.cuh"
 
@@ -186,8 +187,7 @@ size_t smem_frame_r() { return sizeof(float2) * (N + (size_t)N * reg_pitch<N>())
 template <int N>
 void launch_frame(const ProbArgs& a, int form, int upd_probe, cudaStream_t s) {
     if constexpr (frame_whole<N>()) {
-        const int per_sm = N >= 64 ? 2 : 4;
-        const int grid = a.J < per_sm * sm_count() ? a.J : per_sm * sm_count();
+        const int grid = a.J < frame_blocks(N) ? a.J : frame_blocks(N);
         auto k = form == FRAME_DM ? k_frame_r<N, FRAME_DM> : (form == FRAME_LLK ? k_frame_r<N, FRAME_LLK> : k_frame_r<N, FRAME_PHI>);
         k<<<grid, frame_threads<N>(), smem_frame_r<N>(), s>>>(a, upd_probe);
     }
