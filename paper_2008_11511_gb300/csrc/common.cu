@@ -154,7 +154,10 @@ __global__ void k_normalise(ProbArgs a, float alpha_obj, float alpha_probe, int 
 // The probe's max D_P and normalisation in one launch, for probes that one
 // cluster of kProbeCtas blocks holds in registers (K N^2 <= kProbeMax pixels): each
 // thread keeps its pixels' accumulators, the blocks' maxima meet through
-// distributed shared memory.  Replaces k_den_max and k_normalise, two launches
+// distributed shared memory.  A block may only touch another's shared memory once
+// that block has started, which nothing but a cluster barrier says: every thread
+// arrives at entry and waits just before the stores, with the loads of the
+// accumulators in between.  Replaces k_den_max and k_normalise, two launches
 // of 3 to 4 us that each wait for the one before (64^2: 4.0 us, 128^2: 6.5 us in
 // one; at 256^2 eight blocks take 14 us, the two launches 9).
 constexpr int kProbeCtas = 8, kProbeThreads = 512;
@@ -164,6 +167,7 @@ __global__ void __cluster_dims__(kProbeCtas, 1, 1) __launch_bounds__(kProbeThrea
     k_probe_norm(ProbArgs a, float alpha_probe) {
     __shared__ float red[kProbeThreads / 32];
     __shared__ float maxima[kProbeCtas];  // every block's, written by the others
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const int n1 = a.N * a.N, n = a.K * n1;
     const int i0 = blockIdx.x * kProbeThreads + threadIdx.x;
     constexpr int kStep = kProbeCtas * kProbeThreads;
@@ -178,6 +182,7 @@ __global__ void __cluster_dims__(kProbeCtas, 1, 1) __launch_bounds__(kProbeThrea
     mx = warp_max(mx);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
     __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every block has started
     if (threadIdx.x < kProbeCtas) {
         float b = 0.f;
 #pragma unroll
@@ -187,6 +192,7 @@ __global__ void __cluster_dims__(kProbeCtas, 1, 1) __launch_bounds__(kProbeThrea
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(threadIdx.x));
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(b) : "memory");
     }
+    __syncwarp();
     // (after this barrier no block touches another's shared memory)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     float m = 0.f;

@@ -226,3 +226,23 @@ def test_split_passes_gradient(N, K, J, masked, parts):
             assert np.linalg.norm(a.cpu().numpy() - b) <= tol * np.linalg.norm(b)
     assert abs(float(llk) - rl) < 1e-6 * rl
     pb.close()
+
+
+# probes that one cluster holds (one pixel per thread, four, the last size it takes) and the first one beyond
+@pytest.mark.parametrize("N,K", [(8, 1), (12, 3), (32, 4), (64, 1), (64, 3), (128, 1), (80, 3), (128, 2)])
+def test_probe_update_around_the_cluster_limit(N, K):
+    """The probe's denominator maximum and normalisation, one launch up to 16384
+    pixels, against the oracle, over several cycles of the same handle."""
+    from paper_2008_11511_gb300 import Ptycho
+    J = 4
+    obj, probe, pos, psi, io, mask = _scan(N, K, J, True, 30 * K + N)
+    data = oracle.Data.make(io, pos, mask)
+    o, p = dev(obj), dev(probe)
+    pb = Ptycho(o, p, dev(io), pos, mask, psi=dev(psi))
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
+    for _ in range(3):
+        before = p.cpu().numpy()
+        pb.ap(1, update_obj=False)
+        _, rp, _ = oracle.ap_cycle(obj, before.reshape(probe.shape), data, update_obj=False)
+        assert np.linalg.norm(p.cpu().numpy() - rp) < tol * np.linalg.norm(rp)
+    pb.close()
