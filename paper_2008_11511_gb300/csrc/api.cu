@@ -650,10 +650,13 @@ ptx_status compute_layout(std::vector<ProbHost>& probs, size_t* spec_off, size_t
         h.lay.pos_part += o;
         h.lay.end += o;
         o += sz;
-        // at least the three waves per mode of one frame of the line search (more
-        // than the lanes' slices hold when there is a single frame)
+        // the lanes' slices, each of at least one frame for as many lanes as "lanes" can ask
+        // for: a single-frame problem's frame in lane 3 would otherwise end beyond the
+        // stack (and the scratch), and lanes next to each other would share part of it.
+        // It also holds the three waves per mode of one frame of the line search.
         const size_t frame = (size_t)h.p.K * h.p.N * h.p.N * sizeof(float2);
-        spec = std::max(spec, std::max((size_t)h.Bfit * kDefaultLanes, (size_t)3) * frame);
+        static_assert(kMaxLanes >= 3, "three waves of a frame");
+        spec = std::max(spec, std::max((size_t)h.Bfit * kDefaultLanes * frame, kMaxLanes * align_up(frame)));
         frames += (size_t)h.p.J;
     }
     *ctl_off = o;

@@ -112,6 +112,23 @@ def test_work_stack_sizing(lib):
     assert 64 * mb < n512k1 < 96 * mb
 
 
+def test_work_stack_holds_a_frame_for_every_lane(lib):
+    """Single-frame problems: the stack (what a second equal problem does not
+    add to the size) has a frame for each of the four lanes that "lanes" can
+    ask for, so that lanes at work on different problems share none of it."""
+    from paper_2008_11511_gb300._lib import Problem
+    for N, K in ((512, 8), (400, 3), (256, 1), (80, 2)):
+        p, pos = _problem(N=N, K=K, Ho=N + 4, Wo=N + 4, positions=[[1, 2]])
+        size = []
+        for n in (1, 2):
+            out = ctypes.c_size_t(0)
+            assert lib.ptx_workspace_bytes((Problem * n)(*[p] * n), n, ctypes.byref(out)) == 0
+            size.append(out.value)
+        stack = 2 * size[0] - size[1]  # and the control block, a few hundred bytes
+        frame = K * N * N * 8
+        assert 4 * frame <= stack < 4 * frame + 16384, (N, K, stack, frame)
+
+
 def test_encode_counts8_matches_its_definition(lib):
     """ptx_encode_counts8 (host): out8 = min(c, 255), escapes = every index
     with c >= 255 in increasing order with its count; boundaries 254 / 255 /

@@ -211,3 +211,41 @@ def test_persistent_schedule_wait_gives_up_and_reports():
     o, p, _ = oracle.ap_cycle(o0, p0, data)
     assert rel(pb.items[0]["obj"].cpu().numpy(), o) < TOL1
     pb.close()
+
+
+# 12: a frame of 1152 bytes, no multiple of the slices' alignment; 64: without the stack; 160, 256: split passes
+@pytest.mark.parametrize("sizes", [[(12, 1)] * 4, [(80, 1)] * 5, [(160, 2), (256, 1), (64, 1), (256, 2), (160, 1)]])
+@pytest.mark.parametrize("lanes", [1, 3, 4])
+def test_single_frame_problems_in_every_lane(sizes, lanes):
+    """Problems of one frame each, spread over the lanes: every lane has a slice
+    of the work stack for its frame (DM and AP against the oracle)."""
+    from paper_2008_11511_gb300 import PtychoBatch
+    rng = np.random.default_rng(len(sizes) + lanes)
+
+    def crandn(*shape):
+        return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+    items, refs, algos = [], [], []
+    for i, (N, K) in enumerate(sizes):
+        obj, probe = (1 + 0.3 * crandn(N + 3, N + 2)).astype(np.complex64), crandn(K, N, N)
+        pos = np.array([[i % 3, 1]], dtype=np.int32)
+        phi = oracle.obj_probe_to_psi(obj, probe, pos)
+        psi = (phi * (1 + 0.1 * crandn(*phi.shape))).astype(np.complex64)
+        ic = (np.abs(np.fft.fft2(phi, norm="ortho")) ** 2).sum(1)
+        io = (ic * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+        data = oracle.Data.make(io, pos, None)
+        items.append(dict(obj=dev(obj), probe=dev(probe), iobs=dev(io), positions=pos, mask=None, psi=dev(psi)))
+        if i % 2:
+            algos.append("DM")
+            refs.append(oracle.dm_cycle(obj, probe, psi, data)[:2])
+        else:
+            algos.append("AP")
+            refs.append(oracle.ap_cycle(obj, probe, data)[:2])
+    pb = PtychoBatch(items)
+    pb.set_param("lanes", lanes)
+    pb.cycles(1, algos)
+    for (N, _), it, (ro, rp) in zip(sizes, pb.items, refs):
+        # single precision: 4 transforms of log2 N levels and a dozen roundings, each 2^-24 of the rms
+        tol = 2.0 ** -24 * (8 * np.log2(N) + 13)
+        assert rel(it["obj"].cpu().numpy(), ro) < tol and rel(it["probe"].cpu().numpy(), rp) < tol
+    pb.close()
