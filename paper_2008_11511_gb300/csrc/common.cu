@@ -113,38 +113,45 @@ __global__ void k_den_max(ProbArgs a, int upd_obj, int upd_probe) {
 // O <- (N_O + d_O O) / (D_O + d_O), d_O = alpha_obj max D_O (unchanged where the
 // denominator is 0); the same for each probe mode with D_P; accumulators cleared,
 // and by the last block the maxima, which every block has read by then (a memset
-// node per cycle for them took 5 us of a 30 us cycle).
+// node per cycle for them took 5 us of a 30 us cycle).  A block takes its ticket
+// once all its threads have read the maxima, before its first store: a fence
+// behind the stores would wait for them (cycle of 100 x 64^2: 27.0 -> 28.8 us).  The
+// first pixel's loads go out before that barrier.
 __global__ void k_normalise(ProbArgs a, float alpha_obj, float alpha_probe, int upd_obj, int upd_probe) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (upd_obj) {
-        const float d = alpha_obj * __uint_as_float(a.maxbits[0]);
-        const size_t n = (size_t)a.Ho * a.Wo;
-        for (size_t i = i0; i < n; i += stride) {
-            const float4 v = a.acc_obj[i];
-            const float den = v.z + d;
-            if (den > 0.f) {
-                const float2 o = a.obj[i];
-                a.obj[i] = make_float2((v.x + d * o.x) / den, (v.y + d * o.y) / den);
-            }
-            a.acc_obj[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    if (upd_probe) {
-        const float d = alpha_probe * __uint_as_float(a.maxbits[1]);
-        const size_t n = (size_t)a.K * a.N * a.N;
-        for (size_t i = i0; i < n; i += stride) {
-            const float4 v = a.acc_probe[i];
-            const float den = v.z + d;
-            if (den > 0.f) {
-                const float2 o = a.probe[i];
-                a.probe[i] = make_float2((v.x + d * o.x) / den, (v.y + d * o.y) / den);
-            }
-            a.acc_probe[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
+    const size_t no = upd_obj ? (size_t)a.Ho * a.Wo : 0, np = upd_probe ? (size_t)a.K * a.N * a.N : 0;
+    const float d_o = upd_obj ? alpha_obj * __uint_as_float(a.maxbits[0]) : 0.f;
+    const float d_p = upd_probe ? alpha_probe * __uint_as_float(a.maxbits[1]) : 0.f;
+    float4 v;
+    float2 o;
+    auto load = [&](const float4* acc, const float2* x, size_t i) {
+        v = acc[i];
+        o = x[i];
+    };
+    if (i0 < no) load(a.acc_obj, a.obj, i0);
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&a.maxbits[2], 1u) == gridDim.x - 1) {
+    unsigned ticket = 0;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the block's reads of the maxima come before its ticket
+        ticket = atomicAdd(&a.maxbits[2], 1u);
+    }
+    auto store = [&](float4* acc, float2* x, size_t i, float d) {
+        const float den = v.z + d;
+        if (den > 0.f) x[i] = make_float2((v.x + d * o.x) / den, (v.y + d * o.y) / den);
+        acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    for (size_t i = i0; i < no;) {
+        store(a.acc_obj, a.obj, i, d_o);
+        i += stride;
+        if (i < no) load(a.acc_obj, a.obj, i);
+    }
+    for (size_t i = i0; i < np; i += stride) {
+        load(a.acc_probe, a.probe, i);
+        store(a.acc_probe, a.probe, i, d_p);
+    }
+    if (threadIdx.x == 0 && ticket == gridDim.x - 1) {
+        __threadfence();  // every block's reads come before these stores
         if (upd_obj) a.maxbits[0] = 0u;
         if (upd_probe) a.maxbits[1] = 0u;
         a.maxbits[2] = 0u;

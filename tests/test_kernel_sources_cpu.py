@@ -33,3 +33,19 @@ def test_peers_shared_memory_is_touched_after_a_cluster_barrier(path):
         waits = [m.start() for m in CLUSTER_WAIT.finditer(body)]
         assert waits and waits[0] < remote[0], name
         assert waits[-1] > remote[-1], name
+
+
+TICKET = re.compile(r"atomicAdd\((?:ticket|&a\.maxbits\[2\]), 1u\)")
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_last_block_tickets_are_fenced(path):
+    """A block that takes a ticket to find out whether it is the last one has a
+    fence right before it, behind what the others must see done (or read), and
+    the last block one between the ticket and what it does for all."""
+    src = re.sub(r"//[^\n]*", "", open(path).read())
+    for m in TICKET.finditer(src):
+        last_statements = "".join(src[:m.start()].rsplit(";", 2)[1:])
+        assert "__threadfence()" in last_statements, src[m.start() - 200:m.end()]
+        after = src[m.end():].split("__global__")[0]
+        assert "gridDim.x - 1" in after and "__threadfence()" in after, src[m.start():m.end() + 300]
