@@ -92,3 +92,50 @@ def test_background_dm_llk_and_gradient():
     _, g_o, g_p = pb.ml_grad()
     assert rel(g_o.cpu().numpy(), go) < 1e-4 and rel(g_p.cpu().numpy(), gp) < 1e-4
     pb.close()
+
+
+# every column pass that updates a background: without and with the split column
+# transform, M a multiple of 4 and not, one mode and several, the near field's
+FORMS = [(64, 1, 0.0), (80, 2, 0.0), (128, 1, 0.0), (256, 1, 0.0), (400, 1, 0.0), (224, 2, 0.0), (512, 2, 0.0)]
+
+
+def _background_only(io, bg, probe, nearfield=0.0):
+    """One cycle of one frame that updates the background alone: B <- B I_o / (I_c + B)."""
+    from paper_2008_11511_gb300 import Ptycho
+    N = io.shape[-1]
+    obj = np.ones((N, N), dtype=np.complex64)
+    pb = Ptycho(dev(obj), dev(probe), dev(io[None]), np.zeros((1, 2), np.int32), None, background=dev(bg),
+                nearfield=nearfield)
+    pb.ap(1, update_obj=False, update_probe=False, update_background=True)
+    out = pb.background.cpu().numpy()
+    pb.close()
+    return out
+
+
+@pytest.mark.parametrize("N,K,nf", FORMS + [(128, 1, 30.0), (256, 1, 90.0)])
+def test_background_quotient_over_its_range(N, K, nf):
+    """No probe, so I_c = 0 and the updated background is B fl(I_o / B): I_o to
+    a unit in the last place of the quotient and the rounding of the product,
+    from the floor of I_c up to the largest values."""
+    rng = np.random.default_rng(N + K)
+    bg = np.exp(rng.uniform(np.log(1e-30), np.log(3e38), (N, N))).astype(np.float32)
+    bg[0, :8] = [1e-30, 1.1e-30, 1.0, 2.0 ** 126, 2.0 ** 127, 3e38, 1e38, 3.0]
+    io = (bg * np.exp(rng.uniform(np.log(1e-6), 0.0, (N, N)))).astype(np.float32)
+    io[1, :4] = [0.0, -3.0, 0.0, 0.0]
+    got = _background_only(io, bg, np.zeros((K, N, N), np.complex64), nf)
+    want = np.maximum(io, 0.0).astype(np.float64)
+    assert np.all(np.isfinite(got))
+    normal = want >= 2.0 ** -126
+    assert np.all(np.abs(got - want)[normal] <= 2.0 ** -22 * want[normal])
+    assert np.all(got[~normal] <= 2.0 ** -126)
+
+
+@pytest.mark.parametrize("N,K,nf", FORMS)
+def test_background_under_an_infinite_model_intensity(N, K, nf):
+    """A model intensity beyond the range of single precision leaves no
+    background (I_o / inf = 0), as the exact division gives it."""
+    probe = np.zeros((K, N, N), np.complex64)
+    probe[0, 0, 0] = 3.2e19  # |.|^2 is infinite at every detector pixel
+    io = np.full((N, N), 7.0, np.float32)
+    got = _background_only(io, np.full((N, N), 5.0, np.float32), probe)
+    assert np.all(got == 0.0)
