@@ -97,17 +97,19 @@ __global__ void __launch_bounds__(256, 2) k_col_tc(ProbArgs a, int j0, int nb, i
         }
         if (good) {
             // projection and LLK on X^[q + 16 k1] (thread = vector (c, k2 = q))
+            by_brightness(io, [&](auto bright) {
 #pragma unroll
-            for (int k1 = 0; k1 < 16; ++k1) {
-                const float2 X = make_float2(o[2 * k1], o[2 * k1 + 1]);
-                const float ic = cnorm(X) * invN2;
-                const bool masked = (mbits >> k1) & 1u;
-                float ratio;
-                const float term = llk_term_ratio(ic, io[k1], ratio);
-                if (!masked) llk += term;
-                const float f = masked ? 0.f : (ratio - 1.0f) * invN2;
-                v[k1] = cscale(X, f);
-            }
+                for (int k1 = 0; k1 < 16; ++k1) {
+                    const float2 X = make_float2(o[2 * k1], o[2 * k1 + 1]);
+                    const float ic = cnorm(X) * invN2;
+                    const bool masked = (mbits >> k1) & 1u;
+                    float ratio;
+                    const float term = llk_term_ratio<bright.value>(ic, io[k1], ratio);
+                    if (!masked) llk += term;
+                    const float f = masked ? 0.f : (ratio - 1.0f) * invN2;
+                    v[k1] = cscale(X, f);
+                }
+            });
             // inverse stage 1 over k1 on the thread's own vector, then twiddle w^(+k2 kk)
             pp.put_row(v);
             good = pp.stage(1, o);
@@ -210,16 +212,20 @@ __global__ void __launch_bounds__(512, 1) k_col_tc512(ProbArgs a, int j0) {
     KahanF llk;
     if (good) {
         const float* ib = a.iobs + (size_t)j * N * N + x0 + c2;
+        float io[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int row = k2 + 16 * (16 * h + i);
-            const float io = __ldcs(ib + (size_t)row * N);
-            const bool masked = a.mask[(size_t)row * N + x0 + c2] != 0;
-            float ratio;
-            const float term = llk_term_ratio(ic[i] * invN2, io, ratio);
-            if (!masked) llk.add(term);
-            ic[i] = masked ? 0.f : (ratio - 1.0f) * invN2;  // now the factor
-        }
+        for (int i = 0; i < 16; ++i) io[i] = __ldcs(ib + (size_t)(k2 + 16 * (16 * h + i)) * N);
+        by_brightness(io, [&](auto bright) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int row = k2 + 16 * (16 * h + i);
+                const bool masked = a.mask[(size_t)row * N + x0 + c2] != 0;
+                float ratio;
+                const float term = llk_term_ratio<bright.value>(ic[i] * invN2, io[i], ratio);
+                if (!masked) llk.add(term);
+                ic[i] = masked ? 0.f : (ratio - 1.0f) * invN2;  // now the factor
+            }
+        });
     }
     // sweep 2: per mode, the scaled spectrum through the inverse stages
     for (int k = 0; k < K && good; ++k) {

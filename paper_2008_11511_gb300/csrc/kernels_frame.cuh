@@ -25,9 +25,59 @@ __host__ __device__ constexpr int frame_threads() { return N * Plan<N>::R; }
 
 enum FrameForm : int { FRAME_PHI = 0, FRAME_DM = 1, FRAME_LLK = 2 };
 
+// The thread's pixels k = 0 .. M - 1 of a column (rows cn + R k of the detector), whose
+// terms are in the rows of col: their LLK (returned) and, but for FRAME_LLK, the
+// first factor of the inverse transform in u.
+template <int N, int kForm, bool kBright>
+__device__ __forceinline__ float project_frame(const float2* col, float2* u, const float* io, uint32_t mbits) {
+    constexpr int M = Plan<N>::M, P = reg_pitch<N>();
+    constexpr float invN2 = 1.0f / float(N * N);
+#pragma unroll
+    for (int i = 0; i < M; ++i) u[i] = col[i * P];
+    Dft<M, -1>::run(u);
+    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        const float ic = cnorm(u[i]) * invN2;
+        const bool masked = (mbits >> i) & 1u;
+        float ratio;
+        const float term = llk_term_ratio<kBright>(ic, io[i], ratio);
+        if (!masked) llk += term;
+        if constexpr (kForm != FRAME_LLK) u[i] = cscale(u[i], masked ? 0.f : (ratio - 1.0f) * invN2);
+    }
+    if constexpr (kForm != FRAME_LLK) Dft<M, +1>::run(u);
+    return llk;
+}
+template <int N>
+__device__ __forceinline__ void frame_put(float2* col, const float2* u, const float2* tw, int cn) {
+    constexpr int M = Plan<N>::M, P = reg_pitch<N>();
+    col[0] = u[0];
+#pragma unroll
+    for (int i = 1; i < M; ++i) col[i * P] = cmul(u[i], tw_get<N, +1>(tw, cn, i));
+}
+// Both with the scaled quotients, for a thread whose sum is not finite in frame j.
+template <int N, int kForm>
+__device__ __noinline__ float frame_bright(const ProbArgs& a, int j) {
+    constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>();
+    extern __shared__ __align__(16) float2 sm[];
+    const int cn = threadIdx.x / N, c = threadIdx.x - cn * N;
+    float2* col = sm + N + cn * M * P + c;
+    float io[M];
+    float2 u[M];
+    uint32_t mbits = 0u;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        io[i] = a.iobs[((size_t)j * N + cn + R * i) * N + c];
+        mbits |= (a.mask[(cn + R * i) * N + c] != 0) ? (1u << i) : 0u;
+    }
+    const float llk = project_frame<N, kForm, true>(col, u, io, mbits);
+    if constexpr (kForm != FRAME_LLK) frame_put<N>(col, u, sm, cn);
+    return llk;
+}
+
 // grid (blocks): block x handles frames x, x + gridDim.x, ...
 template <int N, int kForm>
-__global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r(ProbArgs a, int upd_probe) {
+__global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r(const __grid_constant__ ProbArgs a, int upd_probe) {
     constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>(), T = frame_threads<N>();
     constexpr bool kWarp = R == M && 32 % R == 0;  // a row's threads are in one warp in both factors
     extern __shared__ __align__(16) float2 sm[];
@@ -58,7 +108,6 @@ __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r
     uint32_t mbits = 0u;  // rows cn + R i of column c
 #pragma unroll
     for (int i = 0; i < M; ++i) mbits |= (a.mask[(cn + R * i) * N + c] != 0) ? (1u << i) : 0u;
-    constexpr float invN2 = 1.0f / float(N * N);
     __syncthreads();
     for (int j = blockIdx.x; j < a.J; j += gridDim.x) {
         const int2 p = a.pos[j];
@@ -107,27 +156,13 @@ __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r
             for (int i = 1; i < R; ++i) buf[(cn + M * i) * P + c] = cmul(v[i], tw_get<N, -1>(tw, i, cn));
         }
         __syncthreads();
-        // columns, second factor: rows cn M + i hold the terms of ky = cn + R k
-#pragma unroll
-        for (int i = 0; i < M; ++i) u[i] = buf[(cn * M + i) * P + c];
-        Dft<M, -1>::run(u);
-        float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            const float ic = cnorm(u[i]) * invN2;
-            const bool masked = (mbits >> i) & 1u;
-            float ratio;
-            const float term = kForm == FRAME_LLK ? llk_term_fast(ic, io[i]) : llk_term_ratio(ic, io[i], ratio);
-            if (!masked) llk += term;
-            if constexpr (kForm != FRAME_LLK) u[i] = cscale(u[i], masked ? 0.f : (ratio - 1.0f) * invN2);
-        }
-        if constexpr (kForm != FRAME_LLK) {
-            // inverse, first factor over k, into the rows just read
-            Dft<M, +1>::run(u);
-            buf[cn * M * P + c] = u[0];
-#pragma unroll
-            for (int i = 1; i < M; ++i) buf[(cn * M + i) * P + c] = cmul(u[i], tw_get<N, +1>(tw, cn, i));
-        }
+        // columns, second factor: rows cn M + i hold the terms of ky = cn + R k; projection and LLK,
+        // first factor of the inverse over k, into the rows just read
+        float llk = project_frame<N, kForm, false>(buf + cn * M * P + c, u, io, mbits);
+        if (!(llk < kInf))  // bright pixels without a model
+            llk = frame_bright<N, kForm>(a, j);
+        else if constexpr (kForm != FRAME_LLK)
+            frame_put<N>(buf + cn * M * P + c, u, tw, cn);
         const double tot = block_sum_pos<T>(llk, red_s);  // also the barrier of the exchange
         if (t == 0) a.llk_part[j] = tot;
         if constexpr (kForm == FRAME_LLK) {

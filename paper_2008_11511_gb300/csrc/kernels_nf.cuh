@@ -170,20 +170,25 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_row_pro
             Dft<M, +1>::run(u[i]);
             const float* io_row = a.iobs + ((size_t)j * N + y) * N + k2;
             const uint8_t* mk_row = a.mask + (size_t)y * N + k2;
+            float io_r[M];
 #pragma unroll
-            for (int k1 = 0; k1 < M; ++k1) {
-                float ic = cnorm(u[i][k1]);
-                const float io = __ldcs(io_row + R * k1);
-                const bool masked = mk_row[R * k1] != 0;
-                if (bgp) {  // incoherent background in the detector plane
-                    const int pix = y * N + k2 + R * k1;
-                    ic += __ldg(bgp + pix);
-                    if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, quotient(io, ic));
+            for (int k1 = 0; k1 < M; ++k1) io_r[k1] = __ldcs(io_row + R * k1);
+            by_brightness(io_r, [&](auto bright) {
+#pragma unroll
+                for (int k1 = 0; k1 < M; ++k1) {
+                    float ic = cnorm(u[i][k1]);
+                    const float io = io_r[k1];
+                    const bool masked = mk_row[R * k1] != 0;
+                    if (bgp) {  // incoherent background in the detector plane
+                        const int pix = y * N + k2 + R * k1;
+                        ic += __ldg(bgp + pix);
+                        if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, quotient(io, ic));
+                    }
+                    if (!masked) llk += llk_term_fast<bright.value>(ic, io);
+                    const float f = masked ? 0.f : amp_ratio(io, ic) - 1.0f;
+                    u[i][k1] = cscale(u[i][k1], f);
                 }
-                if (!masked) llk += llk_term_fast(ic, io);
-                const float f = masked ? 0.f : amp_ratio(io, ic) - 1.0f;
-                u[i][k1] = cscale(u[i][k1], f);
-            }
+            });
             if (!llk_only) {
                 // the correction in natural order, for the forward row FFT
                 float2* o = buf + line * P + k2;

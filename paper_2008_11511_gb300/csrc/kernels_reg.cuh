@@ -118,6 +118,81 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_r(
 #undef PTX_BY
 }
 
+// A thread's M pixels of a column pass (R N apart): their model intensities, the
+// LLK (returned), and the spectrum u scaled by the projection's factor or the
+// gradient's weight.  bg, bg_acc: the background and its sums at pixel k1 = 0.
+template <int N, bool kBg, bool kBright>
+__device__ __forceinline__ float project_pixels(float2* u, const float* io, uint32_t mbits, int mode, const float* bg,
+                                           float* bg_acc, bool add_bg) {
+    constexpr int M = Plan<N>::M, RN = Plan<N>::R * N;
+    constexpr float invN2 = 1.0f / float(N * N);
+    [[maybe_unused]] QuadAdd<M> bg_sum(bg_acc, RN);
+    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        float ic = cnorm(u[k1]) * invN2;
+        const bool masked = (mbits >> k1) & 1u;
+        if constexpr (kBg) {  // incoherent background: one more component of the model intensity
+            ic += __ldg(bg + k1 * RN);
+            if (add_bg) bg_sum.put(k1, masked ? 0.f : quotient(io[k1], ic));
+        }
+        float f;
+        if (mode == COL_PROJECT) {
+            float ratio;
+            const float term = llk_term_ratio<kBright>(ic, io[k1], ratio);
+            if (!masked) llk += term;
+            f = masked ? 0.f : (ratio - 1.0f) * invN2;
+        } else {
+            if (!masked) llk += llk_term_fast<kBright>(ic, io[k1]);
+            f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io[k1], ic)) * invN2;
+        }
+        u[k1] = cscale(u[k1], f);
+    }
+    return llk;
+}
+// The part of the column pass between its two transposes for a thread whose LLK is
+// not finite (block bx, frame by of the batch), with the scaled quotients and
+// without the background's sums, which are in already.  The transposes' buffer is
+// being rewritten, so the terms of the second factor come from the work stack, which
+// is not yet, by their definition.  It takes what it needs from the arguments, so
+// that the pass keeps no register for it.
+template <int N, bool kBg>
+__device__ __noinline__ float col_bright_r(const ProbArgs& a, int j0, int bx, int by, int mode) {
+    using S = RegShape<N>;
+    constexpr int R = S::R, M = S::M, C = S::C, P = S::P;
+    extern __shared__ __align__(16) float2 sm[];
+    const float2* tw = sm;
+    float llk = 0.f;
+    for (int w = threadIdx.x; w < C * R; w += kThreads) {
+        const int k2 = w / C, c = w - k2 * C, pix = k2 * N + bx * C + c;
+        const float* ib = a.iobs + (size_t)(j0 + by) * N * N + pix;
+        const float2* spec = a.spec + (size_t)by * N * N + bx * C + c;
+        float io[M];
+        float2 u[M];
+        uint32_t mbits = 0u;
+        for (int n1 = 0; n1 < M; ++n1) {
+            io[n1] = ib[n1 * R * N];
+            mbits |= (a.mask[pix + n1 * R * N] != 0) ? (1u << n1) : 0u;
+            float2 s = make_float2(0.f, 0.f);
+            for (int n2 = 0; n2 < R; ++n2) {
+                float2 t;  // w_N^(n k2), n = n1 + M n2
+                sincospif(-2.f * (float)((n1 + M * n2) * k2 % N) / (float)N, &t.y, &t.x);
+                s = cadd(s, cmul(spec[(size_t)(n1 + M * n2) * N], t));
+            }
+            u[n1] = s;
+        }
+        Dft<M, -1>::run(u);
+        llk += project_pixels<N, kBg, true>(u, io, mbits, mode, kBg ? a.bg + pix : nullptr, nullptr, false);
+        if (mode != COL_LLK) {
+            Dft<M, +1>::run(u);
+            float2* o = sm + N + c * P + k2;
+            o[0] = u[0];
+            for (int kk = 1; kk < M; ++kk) o[kk * (R + 1)] = cmul(u[kk], tw_get<N, +1>(tw, k2, kk));
+        }
+    }
+    return llk;
+}
+
 // ---------------------------------------------------------------------------
 // Column pass: column FFT, projection + LLK, inverse column FFT.
 // grid (N / L, frames in batch); block handles columns [x0, x0 + L).
@@ -127,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::MinBlocks) k_row_fwd_r(
 // cycle's projection (COL_PROJECT) fixed at compile time; otherwise the mode
 // comes from the argument.
 template <int N, bool kBg, bool kCycle>
-__global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_r(ProbArgs a, int j0, int mode_arg) {
+__global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_r(const __grid_constant__ ProbArgs a, int j0, int mode_arg) {
 #define PTX_BX blockIdx.x
 #define PTX_BY blockIdx.y
 #define PTX_GX gridDim.x
@@ -236,28 +311,33 @@ __global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_mod
             if (a.mbits) mbits = a.mbits[blockIdx.x * kThreads + threadIdx.x] >> (i * M);
             const float* ib = a.iobs + (size_t)j * N * N + (size_t)k2 * N + x0 + c;
             QuadAdd<M> bg_sum(a.bg_acc + (size_t)k2 * N + x0 + c, R * N);
+            float io_r[M];
 #pragma unroll
-            for (int k1 = 0; k1 < M; ++k1) {
-                const int pix = (k2 + R * k1) * N + x0 + c;
-                const bool masked = a.mbits ? ((mbits >> k1) & 1u) != 0u : a.mask[pix] != 0;
-                float ic = ic_r[i][k1] * invN2;
-                const float io = __ldcs(ib + (size_t)R * k1 * N);
-                if (bgp) {
-                    ic += __ldg(bgp + pix);
-                    if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
+            for (int k1 = 0; k1 < M; ++k1) io_r[k1] = __ldcs(ib + (size_t)R * k1 * N);
+            by_brightness(io_r, [&](auto bright) {
+#pragma unroll
+                for (int k1 = 0; k1 < M; ++k1) {
+                    const int pix = (k2 + R * k1) * N + x0 + c;
+                    const bool masked = a.mbits ? ((mbits >> k1) & 1u) != 0u : a.mask[pix] != 0;
+                    float ic = ic_r[i][k1] * invN2;
+                    const float io = io_r[k1];
+                    if (bgp) {
+                        ic += __ldg(bgp + pix);
+                        if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
+                    }
+                    float f;
+                    if (mode == COL_PROJECT) {
+                        float ratio;
+                        const float term = llk_term_ratio<bright.value>(ic, io, ratio);
+                        if (!masked) llk += term;
+                        f = masked ? 0.f : (ratio - 1.0f) * invN2;
+                    } else {
+                        if (!masked) llk += llk_term_fast<bright.value>(ic, io);
+                        f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
+                    }
+                    ic_r[i][k1] = f;
                 }
-                float f;
-                if (mode == COL_PROJECT) {
-                    float ratio;
-                    const float term = llk_term_ratio(ic, io, ratio);
-                    if (!masked) llk += term;
-                    f = masked ? 0.f : (ratio - 1.0f) * invN2;
-                } else {
-                    if (!masked) llk += llk_term_fast(ic, io);
-                    f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
-                }
-                ic_r[i][k1] = f;
-            }
+            });
         }
     }
     const double tot = block_sum_pos<kThreads>(llk, red_s);

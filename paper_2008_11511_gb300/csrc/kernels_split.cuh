@@ -114,11 +114,38 @@ __global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_row_fwd_
 #undef PTX_DST
 }
 
+// k_col_s for a warp with a thread whose LLK is not finite, again from and back to the work
+// stack (which still holds the values): with the scaled quotients, and without the
+// background's sums, which are in already.  It takes what it needs from the kernel's
+// parameters, so that k_col_s keeps no register for it.
+template <int N, bool kBg>
+__device__ __noinline__ float col_bright_s(const ProbArgs& a, int j0, int mode) {
+    constexpr int M = Plan<N>::M, RN = Plan<N>::R * N;
+    const int id = blockIdx.x * SplitShape<N>::TC + threadIdx.x;
+    const float* ib = a.iobs + (size_t)(j0 + blockIdx.y) * N * N + id;
+    float2* spec = a.spec + (size_t)blockIdx.y * N * N + id;
+    float io[M];
+    float2 u[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) {
+        io[k1] = ib[k1 * RN];
+        u[k1] = spec[k1 * RN];
+    }
+    Dft<M, -1>::run(u);
+    const float llk = project_pixels<N, kBg, true>(u, io, a.mbits_s[id], mode, kBg ? a.bg + id : nullptr, nullptr, false);
+    if (mode != COL_LLK) {
+        Dft<M, +1>::run(u);
+#pragma unroll
+        for (int n1 = 0; n1 < M; ++n1) spec[n1 * RN] = u[n1];
+    }
+    return llk;
+}
+
 // Column pass, one mode: second factor, projection and LLK (or the gradient's
 // weights), second factor of the inverse.  grid (N / C, frames in batch)
 template <int N, bool kBg, bool kCycle>
 __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * kThreads / SplitShape<N>::TC)
-    k_col_s(ProbArgs a, int j0, int mode_arg) {
+    k_col_s(const __grid_constant__ ProbArgs a, int j0, int mode_arg) {
     const int mode = kCycle ? (int)COL_PROJECT : mode_arg;
     using S = SplitShape<N>;
     constexpr int R = S::R, M = S::M, RN = R * N;
@@ -139,34 +166,15 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
 #pragma unroll
     for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + n1 * RN, el);
     Dft<M, -1>::run(u);
-    constexpr float invN2 = 1.0f / float(N * N);
-    [[maybe_unused]] QuadAdd<M> bg_sum(a.bg_acc + id, RN);
-    float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+    float llk = project_pixels<N, kBg, false>(u, io, mbits, mode, kBg ? a.bg + id : nullptr, a.bg_acc + id, a.bg_acc != nullptr);
+    if (__all_sync(0xffffffffu, llk < kInf)) {
+        if (mode != COL_LLK) {
+            Dft<M, +1>::run(u);
 #pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) {
-        float ic = cnorm(u[k1]) * invN2;
-        const bool masked = (mbits >> k1) & 1u;
-        if constexpr (kBg) {  // incoherent background: one more component of the model intensity
-            const int pix = id + k1 * RN;
-            ic += __ldg(a.bg + pix);
-            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io[k1], ic));
+            for (int n1 = 0; n1 < M; ++n1) st_hint(spec + n1 * RN, u[n1], el);
         }
-        float f;
-        if (mode == COL_PROJECT) {
-            float ratio;
-            const float term = llk_term_ratio(ic, io[k1], ratio);
-            if (!masked) llk += term;
-            f = masked ? 0.f : (ratio - 1.0f) * invN2;
-        } else {
-            if (!masked) llk += llk_term_fast(ic, io[k1]);
-            f = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io[k1], ic)) * invN2;
-        }
-        u[k1] = cscale(u[k1], f);
-    }
-    if (mode != COL_LLK) {
-        Dft<M, +1>::run(u);
-#pragma unroll
-        for (int n1 = 0; n1 < M; ++n1) st_hint(spec + n1 * RN, u[n1], el);
+    } else {  // bright pixels without a model
+        llk = col_bright_s<N, kBg>(a, j0, mode);
     }
     const double tot = block_sum_pos<S::TC>(llk, red_s);
     if (threadIdx.x == 0) a.llk_part[(size_t)j * gridDim.x + blockIdx.x] = tot;
@@ -207,26 +215,31 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
     const float* ib = a.iobs + (size_t)j * N * N + id;
     QuadAdd<M> bg_sum(a.bg_acc + id, RN);
     float llk = 0.f;  // the terms are >= 0: a plain float sum of a thread's pixels
+    float io_r[M];
 #pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) {
-        const bool masked = (mbits >> k1) & 1u;
-        const float io = __ldcs(ib + k1 * RN);
-        float ic = f[k1] * invN2;
-        if (bgp) {
-            const int pix = id + k1 * RN;
-            ic += __ldg(bgp + pix);
-            if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
+    for (int k1 = 0; k1 < M; ++k1) io_r[k1] = __ldcs(ib + k1 * RN);
+    by_brightness(io_r, [&](auto bright) {
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1) {
+            const bool masked = (mbits >> k1) & 1u;
+            const float io = io_r[k1];
+            float ic = f[k1] * invN2;
+            if (bgp) {
+                const int pix = id + k1 * RN;
+                ic += __ldg(bgp + pix);
+                if (a.bg_acc) bg_sum.put(k1, masked ? 0.f : quotient(io, ic));
+            }
+            if (mode == COL_PROJECT) {
+                float ratio;
+                const float term = llk_term_ratio<bright.value>(ic, io, ratio);
+                if (!masked) llk += term;
+                f[k1] = masked ? 0.f : (ratio - 1.0f) * invN2;
+            } else {
+                if (!masked) llk += llk_term_fast<bright.value>(ic, io);
+                f[k1] = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
+            }
         }
-        if (mode == COL_PROJECT) {
-            float ratio;
-            const float term = llk_term_ratio(ic, io, ratio);
-            if (!masked) llk += term;
-            f[k1] = masked ? 0.f : (ratio - 1.0f) * invN2;
-        } else {
-            if (!masked) llk += llk_term_fast(ic, io);
-            f[k1] = masked ? 0.f : 2.0f * (1.0f - io_over_ic(io, ic)) * invN2;
-        }
-    }
+    });
     if (mode != COL_LLK) {
         for (int k = 0; k < K; ++k) {
             float2 u[M];
@@ -338,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, SplitShape<N>::ColBlocks) k_row_proj
             ic += __ldg(bgp + pix);
             if (a.bg_acc && !masked) atomicAdd(a.bg_acc + pix, quotient(io[k1], ic));
         }
-        if (!masked) llk += llk_term_fast(ic, io[k1]);
+        if (!masked) llk += llk_term_fast<true>(ic, io[k1]);
         const float f = masked ? 0.f : amp_ratio(io[k1], ic) - 1.0f;
         u[k1] = cscale(u[k1], f);
     }

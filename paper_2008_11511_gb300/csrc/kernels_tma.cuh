@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int k1 = 0; k1 < M; ++k1) {
             const float ic = cnorm(u[k1]) * invN2;
             const bool masked = (mbits >> k1) & 1u;
-            if (!masked) llk.add(llk_term_fast(ic, io[k1]));
+            if (!masked) llk.add(llk_term_fast<true>(ic, io[k1]));
             const float f = masked ? 0.f : (amp_ratio(io[k1], ic) - 1.0f) * invN2;
             u[k1] = cscale(u[k1], f);
         }

@@ -246,3 +246,41 @@ def test_probe_update_around_the_cluster_limit(N, K):
         _, rp, _ = oracle.ap_cycle(obj, before.reshape(probe.shape), data, update_obj=False)
         assert np.linalg.norm(p.cpu().numpy() - rp) < tol * np.linalg.norm(rp)
     pb.close()
+
+
+# whole frames, the unsplit and the split passes, one mode and several, the near field
+BRIGHT = [(12, 1, 0.0), (64, 1, 0.0), (80, 2, 0.0), (128, 1, 0.0), (224, 1, 0.0), (256, 1, 0.0), (256, 3, 0.0), (400, 1, 0.0),
+          (128, 1, 30.0), (256, 1, 90.0)]
+
+
+@pytest.mark.parametrize("N,K,nf", BRIGHT)
+def test_llk_of_bright_pixels_without_a_model(N, K, nf):
+    """The likelihood of counts up to 1e13 where the model intensity is at its
+    floor, 1e-30: I_o / I_c goes far beyond 2^126."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N)
+    io = np.exp(rng.uniform(np.log(1e5), np.log(1e13), (2, N, N))).astype(np.float32)
+    pb = Ptycho(dev(np.ones((N, N), np.complex64)), torch.zeros((K, N, N), dtype=torch.complex64, device="cuda"), dev(io),
+                np.zeros((2, 2), np.int32), None, nearfield=nf)
+    ref = oracle.llk_terms(np.zeros(io.shape), io.astype(np.float64), np.zeros((N, N), bool)).sum()
+    # a term's logarithm is good to a few units of 2^-24 of its size
+    assert abs(float(pb.llk()) - ref) < 2.0 ** -20 * ref
+    pb.close()
+
+
+@pytest.mark.parametrize("N,K", [(n, k) for n, k, nf in BRIGHT if not nf])
+def test_projection_of_a_faint_wave_on_bright_pixels(N, K):
+    """A wave of intensity 1e-29 everywhere takes the amplitude of 1e11 counts: a
+    factor of 1e20 (a probe of one pixel, so that every value is known)."""
+    from paper_2008_11511_gb300 import Ptycho
+    probe = np.zeros((K, N, N), np.complex64)
+    probe[K - 1, 0, 0] = N * np.sqrt(1e-29)
+    io = np.full((1, N, N), 1e11, np.float32)
+    pb = Ptycho(dev(np.ones((N, N), np.complex64)), dev(probe), dev(io), np.zeros((1, 2), np.int32), None)
+    llk = float(pb.ap(1, update_obj=False, update_probe=False)[0])
+    psi = pb.psi.cpu().numpy()[0, K - 1]
+    want = N * np.sqrt(1e11)
+    assert abs(psi[0, 0] - want) < 2.0 ** -20 * want
+    ref = N * N * oracle.llk_terms(np.array([1e-29]), np.array([1e11]), np.zeros(1, bool))[0]
+    assert abs(llk - ref) < 2.0 ** -20 * ref
+    pb.close()
