@@ -494,9 +494,8 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, k
         if ((mbits >> k1) & 1u) continue;
         ic += a.bg ? __ldg(a.bg + id + k1 * RN) : 0.f;
         const float io = fmaxf(__ldcs(io_p + k1 * RN), 0.f);
-        const float ric = rcp_ftz(fmaxf(ic, 1e-30f));  // 1 / I_c (a few ulp)
-        const float w1 = fmaf(-io, ric, 1.f);
-        const float q = di * ric;  // I_o dI^2 / I_c^2 = I_o q^2
+        float w1, q;  // I_o dI^2 / I_c^2 = I_o q^2
+        ls_weights<kModes>(io, ic, di, w1, q);
         l1.add(w1 * di);
         l2.add(fmaf(w1, dd, io * q * q));
     }

@@ -284,3 +284,24 @@ def test_projection_of_a_faint_wave_on_bright_pixels(N, K):
     ref = N * N * oracle.llk_terms(np.array([1e-29]), np.array([1e11]), np.zeros(1, bool))[0]
     assert abs(llk - ref) < 2.0 ** -20 * ref
     pb.close()
+
+
+@pytest.mark.parametrize("N,K", [(32, 2), (64, 3), (128, 2), (256, 3), (512, 2)])
+def test_line_coeffs_vanish_on_exact_intensities(N, K):
+    """Several modes on intensities that equal the model's exactly: I_o / I_c is 1
+    to the last bit by division, so L'(0) is 0.  Probes of one pixel each, and an
+    object of small integers, make every model value exact."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N * K)
+    J = 12
+    obj = rng.integers(1, 8, (N + 3, N + J)).astype(np.complex64)
+    probe = np.zeros((K, N, N), np.complex64)
+    probe[:, 0, 0] = N * np.arange(1, K + 1)  # |P_k O|^2 / N^2 = (k o)^2 at every detector pixel
+    pos = np.stack([np.zeros(J), np.arange(J)], 1).astype(np.int32)
+    ic = (np.arange(1, K + 1) ** 2).sum() * np.abs(obj[0, :J]) ** 2
+    io = np.broadcast_to(ic[:, None, None], (J, N, N)).astype(np.float32)
+    d_o = (1 + rng.random((N + 3, N + J))).astype(np.complex64)
+    pb = Ptycho(dev(obj), dev(probe), dev(io), pos, None, with_psi=False)
+    l1, l2 = pb.line_coeffs(dev(d_o), None).cpu().numpy()
+    pb.close()
+    assert l1 == 0.0 and l2 > 0.0
