@@ -12,8 +12,7 @@
 namespace ptx {
 
 namespace {
-constexpr int kPosSum = 8;             // rows summed in FP32 by a thread
-constexpr int kPosRows = 2 * kPosSum;  // rows each thread walks down
+constexpr int kPosRows = 16;  // rows each thread walks down
 // pairs of adjacent columns, and rows of such pairs a block of 256 threads holds
 __host__ __device__ inline int pos_groups(int N) { return 256 / (N / 2); }
 }  // namespace
@@ -32,23 +31,27 @@ int pos_bands(int N) {
 // pixel is loaded for its own row only (and twice for the neighbours'
 // columns), the probe and the exit wave by 16-byte loads, and no index is
 // divided inside the loop.  With |G|^2 = |P|^2 |dO|^2 and Re(conj(P dO) chi) =
-// Re(conj(dO) w), w = sum_k conj(P_k) Psi_k - |P|^2 O, a mode costs one complex
-// product and |P|^2 instead of three products and five sums.
-// A thread's sums over kPosSum rows stay in FP32, the block's are FP64.
+// Re(conj(dO) w), w = sum_k conj(P_k) chi_k, a mode costs two complex products and
+// |P|^2 instead of three products and five sums.  (chi = Psi - P O comes first: in
+// conj(P) Psi - |P|^2 O the rounding of two large products remains where Psi is
+// near P O.)
+// A thread's sums stay in FP32, with compensation (plain ones would be longer than
+// the 8 N / 256 pixels that a thread added before), the block's are FP64.
 // Sixteen rows per thread re-read 2 halo rows in 18 (8 rows: 2 in 10), and four
 // blocks per SM leave the registers for four rows of loads in flight.
-// 1000 frames of 256^2, all three launches: 1108 -> 203 us (start: every product
+// 1000 frames of 256^2, all three launches: 1108 -> 215 us (before: every product
 // from global memory, FP64 shuffles in every warp, one block for all the solves);
-// 8 rows per thread 213, 32 rows 177 but with longer FP32 sums than before.
+// 203 with plain sums of 16 pixels and the large products, at errors against 64 bits
+// of 6.5 to 7.8e-7 over 64^2 to 512^2 instead of 5.4 to 6.5e-7, as before.
 template <bool kOneMode>
 __global__ void __launch_bounds__(256, kOneMode ? 4 : 3) k_pos_sums(ProbArgs a, double* part) {
-    __shared__ float part_s[2][5][256];
+    __shared__ float part_s[5][256];
     const int N = a.N, K = a.K;
     const int j = blockIdx.x, band = blockIdx.y;
     const int pairs = N / 2, groups = pos_groups(N);
     const int grp = threadIdx.x / pairs, x = 2 * (threadIdx.x - grp * pairs);
     const int y_first = (band * groups + grp) * kPosRows;
-    float s[2][5] = {};  // per half of the rows: yy, yx, xx, y.chi, x.chi
+    KahanF s[5];  // yy, yx, xx, y.chi, x.chi
     if (grp < groups && y_first < N) {
         const int2 p = a.pos[j];
         const int c = p.y + x;                                       // object columns c, c + 1
@@ -63,10 +66,8 @@ __global__ void __launch_bounds__(256, kOneMode ? 4 : 3) k_pos_sums(ProbArgs a, 
         const float2* psi = a.psi + (size_t)j * K * N * N + f0;
         const float2* pr = a.probe + f0;
         const int rows = min(kPosRows, N - y_first);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
 #pragma unroll 4
-          for (int i = h * kPosSum; i < min(rows, (h + 1) * kPosSum); ++i) {
+        for (int i = 0; i < rows; ++i) {
             const bool last = r + i + 1 >= a.Ho, first = r + i == 0;
             const float2* down = last ? row : row + a.Wo;
             const float2 nl = down[cl], n0 = down[c], n1 = down[c + 1], nh = down[cr];
@@ -78,39 +79,37 @@ __global__ void __launch_bounds__(256, kOneMode ? 4 : 3) k_pos_sums(ProbArgs a, 
                 const size_t o = (size_t)k * N * N + (size_t)i * N;
                 const float4 q = __ldg(reinterpret_cast<const float4*>(pr + o));
                 const float4 v = __ldcs(reinterpret_cast<const float4*>(psi + o));
+                const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+                const float2 chi0 = csub(make_float2(v.x, v.y), cmul(q0, o0));
+                const float2 chi1 = csub(make_float2(v.z, v.w), cmul(q1, o1));
                 p0 = fmaf(q.x, q.x, fmaf(q.y, q.y, p0));
                 p1 = fmaf(q.z, q.z, fmaf(q.w, q.w, p1));
-                w0 = cadd(w0, cconjmul(make_float2(q.x, q.y), make_float2(v.x, v.y)));
-                w1 = cadd(w1, cconjmul(make_float2(q.z, q.w), make_float2(v.z, v.w)));
+                w0 = cadd(w0, cconjmul(q0, chi0));
+                w1 = cadd(w1, cconjmul(q1, chi1));
             }
             const float2 gy0 = cscale(csub(n0, m0), sy), gx0 = cscale(csub(o1, ol), sx0);
             const float2 gy1 = cscale(csub(n1, m1), sy), gx1 = cscale(csub(oh, o0), sx1);
-            w0 = make_float2(fmaf(-p0, o0.x, w0.x), fmaf(-p0, o0.y, w0.y));
-            w1 = make_float2(fmaf(-p1, o1.x, w1.x), fmaf(-p1, o1.y, w1.y));
-            s[h][0] = fmaf(p0, cnorm(gy0), fmaf(p1, cnorm(gy1), s[h][0]));
-            s[h][1] = fmaf(p0, fmaf(gy0.x, gx0.x, gy0.y * gx0.y), fmaf(p1, fmaf(gy1.x, gx1.x, gy1.y * gx1.y), s[h][1]));
-            s[h][2] = fmaf(p0, cnorm(gx0), fmaf(p1, cnorm(gx1), s[h][2]));
-            s[h][3] += fmaf(gy0.x, w0.x, fmaf(gy0.y, w0.y, fmaf(gy1.x, w1.x, gy1.y * w1.y)));
-            s[h][4] += fmaf(gx0.x, w0.x, fmaf(gx0.y, w0.y, fmaf(gx1.x, w1.x, gx1.y * w1.y)));
+            s[0].add(fmaf(p0, cnorm(gy0), p1 * cnorm(gy1)));
+            s[1].add(fmaf(p0, fmaf(gy0.x, gx0.x, gy0.y * gx0.y), p1 * fmaf(gy1.x, gx1.x, gy1.y * gx1.y)));
+            s[2].add(fmaf(p0, cnorm(gx0), p1 * cnorm(gx1)));
+            s[3].add(fmaf(gy0.x, w0.x, fmaf(gy0.y, w0.y, fmaf(gy1.x, w1.x, gy1.y * w1.y))));
+            s[4].add(fmaf(gx0.x, w0.x, fmaf(gx0.y, w0.y, fmaf(gx1.x, w1.x, gx1.y * w1.y))));
             m0 = o0; m1 = o1;
             ol = nl; o0 = n0; o1 = n1; oh = nh;
             row = down;
-          }
         }
     }
     // FP64 across the threads: warp q < 5 adds product q of all of them (one
     // FP64 addition per value; shuffling FP64 sums in every warp took 100 us
     // more at 1000 x 256^2, FP64 throughput being a few lanes per clock)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int q = 0; q < 5; ++q) part_s[h][q][threadIdx.x] = s[h][q];
+    for (int q = 0; q < 5; ++q) part_s[q][threadIdx.x] = s[q].s;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp < 5) {
         double v = 0.0;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v += (double)part_s[i >> 3][warp][lane + 32 * (i & 7)];
+        for (int i = 0; i < 8; ++i) v += (double)part_s[warp][lane + 32 * i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if (lane == 0) part[((size_t)j * gridDim.y + band) * 5 + warp] = v;

@@ -89,3 +89,51 @@ def test_refinement_recovers_perturbed_positions():
     err = np.abs(pb.positions - s.positions).sum()
     assert err0 > 20 and err <= err0 // 10, (err0, err)
     pb.close()
+
+
+def _shifts(obj, probe, psi, pos):
+    from paper_2008_11511_gb300 import Ptycho
+    J, N = len(pos), probe.shape[-1]
+    pb = Ptycho(dev(obj), dev(probe), torch.zeros((J, N, N), device="cuda"), pos, psi=dev(psi))
+    d = pb.position_shifts(0.0).cpu().numpy()
+    pb.close()
+    return d
+
+
+@pytest.mark.parametrize("N", [32, 64, 128, 256])
+def test_position_sums_keep_small_terms(N):
+    """A probe of one row in eight, and of so little in the others that a row adds
+    0.4 units in the last place of a bright one: long plain sums lose those rows,
+    3.3e-7 of the norm."""
+    obj = (np.arange(N + 2)[:, None] + 1j * np.arange(N + 2)[None, :]).astype(np.complex64)  # dO/dy = 1, dO/dx = i
+    pos = np.array([[0, 0], [1, 2]], dtype=np.int32)
+    row = np.where(np.arange(N) % 8 == 0, 1.0, np.sqrt(0.4 * 2.0 ** -23))
+    probe = np.broadcast_to(row[None, :, None], (1, N, N)).astype(np.complex64)
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)
+    chi = np.where(np.arange(N) % 8 == 0, 1.0, 0.0)[None, None, :, None] * (0.25 + 0.5j)  # exact sums of the right side
+    psi = (phi + chi).astype(np.complex64)
+    got = _shifts(obj, probe, psi, pos)
+    ref = oracle.position_shifts(obj, probe, psi, pos, 0.0)
+    # a thread's sum rounded once, and the shift itself
+    assert np.abs(got / ref - 1).max() <= 2.0 ** -23
+
+
+@pytest.mark.parametrize("N,K", [(32, 1), (64, 3), (256, 1)])
+def test_position_shifts_near_convergence(N, K):
+    """Exit waves a few units in the last place from P O, all exactly
+    representable: the residual is exact, so the shifts keep their precision."""
+    rng = np.random.default_rng(N + K)
+
+    def ints(m, *shape):
+        return (rng.integers(-m, m + 1, shape) + 1j * rng.integers(-m, m + 1, shape)).astype(np.complex64)
+
+    J = 20
+    obj, probe = ints(511, N + 9, N + 5), ints(127, K, N, N)
+    pos = np.stack([rng.integers(0, 10, J), rng.integers(0, 6, J)], 1).astype(np.int32)
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)  # |Re|, |Im| < 2^17
+    psi = (phi + ints(16, *phi.shape) / 16).astype(np.complex64)
+    got = _shifts(obj, probe, psi, pos)
+    ref = oracle.position_shifts(obj, probe, psi, pos, 0.0)
+    # the right side is a sum of N^2 K terms of random sign, each good to a few units of 2^-24: so is the shift,
+    # to a few units of 2^-24 of its size over the frames
+    assert np.abs(got - ref).max() < 2.0 ** -20 * np.abs(ref).max()
