@@ -369,11 +369,19 @@ void set_batch(ProbHost& h, size_t spec_bytes, int lanes, int cap = 0, int slots
     const int resident = per_sm * sm_count();
     const int rowblk = p.N / h.L3 * p.K;
     int G = slots > 0 ? slots : resident / rowblk;
-    // (DM cycles: 150 x 512^2, 4 / 6 / 9 slots 625 / 620 / 631 us, 203 x 400^2, 6 / 8 / 12: 642 / 638 / 644; 4000 x
-    // 256^2, 19 / 16 / 12: 3193 / 3145 / 3121, which would regroup the probe's sums for 2 %)
-    // the split passes of several modes above 256^2 have half the row blocks: 300 three-mode 512^2 frames, 1 / 2 / 3
-    // slots: 4152 / 3710 / 3647 us
-    if (slots == 0 && p.K > 1 && h.ks->col_s && h.ks->M > h.ks->R) G = 2 * sm_count() / (h.ks->M * p.K);
+    // The split backward pass above 256^2 has M row blocks, half of these, two per SM.
+    // Several modes, one lane, a single batch and batches with a frame or less to a slot
+    // take the slots that fill the GPU so; between two lanes' larger batches of one
+    // mode the old count leaves room for the other lane.
+    //   us per call, old count -> filling: gradient of 60 x 384^2 173 -> 140, 60 x 512^2 320 -> 237;
+    //   cycles in one lane, 100 x 512^2 604 -> 468; 300 three-mode 512^2 frames 4152 -> 3647;
+    //   two lanes, 20 x 384^2 88 -> 77, 16 x 512^2 123 -> 101, but 60 x 384^2 176 -> 180
+    // (at 256^2, 4000 frames, 19 / 16 / 12 slots: 3193 / 3145 / 3121 us, which would
+    // regroup the probe's sums for 2 %)
+    if (slots == 0 && h.ks->col_s && h.ks->M > h.ks->R) {
+        const int full = 2 * sm_count() / (h.ks->M * p.K);
+        if (lanes == 1 || p.K > 1 || h.B <= full || h.B >= p.J) G = full;
+    }
     if (G > h.B) G = h.B;
     if (G < 1) G = 1;
     h.G3 = G;
@@ -728,6 +736,15 @@ bool pass_pdl(const ptx_handle* h, const ProbHost& ph) {
 
 // Whether a problem's passes are those with the column transform split between them.
 bool split_passes(const ProbHost& ph) { return ph.ks->col_s && (ph.p.nearfield <= 0.0 || ph.ks->split_nf); }
+// Whether a cycle's are: not for a few large frames of one mode, whose split row
+// passes, with M blocks per frame instead of N / 8, leave SMs without a block.  DM cycle,
+// unsplit / split: 4 x 384^2 43.6 / 49.5 us, 8 x 384^2 52.9 / 53.6, 10 x 384^2 55.8 / 55.4,
+// 6 x 512^2 64.1 / 67.8, 8 x 512^2 66.1 / 67.2, 11 x 512^2 84.7 / 84.6; two modes gain from the
+// split passes from one frame on (384^2 48.0 / 45.9), 256^2 from four.
+bool split_cycle(const ProbHost& ph) {
+    const bool few = ph.p.K == 1 && ph.ks->M > ph.ks->R && (size_t)ph.p.J * ph.ks->M < (size_t)sm_count() * 4 / 3;
+    return split_passes(ph) && !few;
+}
 
 // The near field's three passes between the forward and the backward row pass:
 // propagate (0), project at the detector (1), propagate back (2).
@@ -1024,7 +1041,7 @@ ptx_status enqueue_cycle(ptx_handle* h, const std::vector<int>& algos, uint32_t 
         // lane's blocks cost more than they save, 20.15 -> 20.21 ms at 512^2, K = 3)
         const bool pdl = pass_pdl(h, ph) && !tc_col && ph.p.K == 1;
         const bool tma_col = h->tma && ph.tma_io && ks->col_tma && ph.p.nearfield <= 0.0 && !ph.p.background;
-        const bool split = split_passes(ph) && !tc_col && !tma_col;
+        const bool split = split_cycle(ph) && !tc_col && !tma_col;
         // (every frame at once: with more, a block's probe sums would run over frames of several batches, and the
         // rounding of sums grouped otherwise grows from cycle to cycle near the waves' zeros: 2453 frames of 64^2,
         // three DM cycles, Psi off by 2.7e-5 of its norm for 8 % of the time)

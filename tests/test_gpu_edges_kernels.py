@@ -305,3 +305,25 @@ def test_line_coeffs_vanish_on_exact_intensities(N, K):
     l1, l2 = pb.line_coeffs(dev(d_o), None).cpu().numpy()
     pb.close()
     assert l1 == 0.0 and l2 > 0.0
+
+
+# the last frame count of the unsplit passes and the first of the split ones; single batches and batches of several lanes
+@pytest.mark.parametrize("N,J", [(384, 8), (384, 9), (400, 8), (400, 9), (448, 7), (448, 8), (512, 6), (512, 7), (512, 16)])
+@pytest.mark.parametrize("lanes,batch", [(1, 0), (2, 0), (2, 4)])
+def test_large_frames_around_the_split_limit(N, J, lanes, batch):
+    """DM cycle of one mode: the choice of the passes by the number of frames, and
+    the backward pass's slots for one lane, one batch and several batches."""
+    from paper_2008_11511_gb300 import Ptycho
+    obj, probe, pos, psi, io, mask = _scan(N, 1, J, True, N + J)
+    data = oracle.Data.make(io, pos, mask)
+    o, p = dev(obj), dev(probe)
+    pb = Ptycho(o, p, dev(io), pos, mask, psi=dev(psi))
+    pb.set_param("lanes", lanes)
+    pb.set_param("batch_frames", batch)
+    llk = pb.dm(1).cpu().numpy()
+    ro, rp, rpsi, rl = oracle.dm_cycle(obj, probe, psi, data)
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
+    for a, b in ((o, ro), (p, rp), (pb.psi, rpsi)):
+        assert np.linalg.norm(a.cpu().numpy() - b) <= tol * np.linalg.norm(b)
+    assert abs(llk[0] - rl) < 1e-6 * rl
+    pb.close()
