@@ -183,66 +183,68 @@ struct ProbHost {
     bool tma_gather = false;
 };
 
-// Tiles of TW x TH object pixels met by at least one frame (pairs: frames per
-// tile summed over the tiles).
-size_t active_tiles(const ptx_problem& p, const int32_t* positions, int TW, int TH, size_t* pairs = nullptr) {
+// The tiles of TW x TH object pixels met by at least one frame, the frames per tile
+// summed over them, and the most frames that one of them has.
+struct TileLoad {
+    size_t tiles = 0, pairs = 0;
+    int longest = 0;
+};
+TileLoad tile_load(const ptx_problem& p, const int32_t* positions, int TW, int TH) {
     const int ntx = (p.Wo + TW - 1) / TW, nty = (p.Ho + TH - 1) / TH;
-    std::vector<char> hit((size_t)ntx * nty, 0);
+    std::vector<int> frames((size_t)ntx * nty, 0);
     for (int j = 0; j < p.J; ++j) {
         const int r = positions[2 * j], c = positions[2 * j + 1];
         for (int ty = r / TH; ty <= (r + p.N - 1) / TH; ++ty)
-            for (int tx = c / TW; tx <= (c + p.N - 1) / TW; ++tx) hit[(size_t)ty * ntx + tx] = 1;
+            for (int tx = c / TW; tx <= (c + p.N - 1) / TW; ++tx) ++frames[(size_t)ty * ntx + tx];
     }
-    size_t n = 0;
-    for (char v : hit) n += v;
-    if (pairs) {
-        *pairs = 0;
-        for (int j = 0; j < p.J; ++j) {
-            const int r = positions[2 * j], c = positions[2 * j + 1];
-            *pairs += (size_t)((r + p.N - 1) / TH - r / TH + 1) * ((c + p.N - 1) / TW - c / TW + 1);
-        }
+    TileLoad load;
+    for (int f : frames) {
+        load.tiles += f > 0;
+        load.pairs += f;
+        load.longest = std::max(load.longest, f);
     }
-    return n;
+    return load;
 }
 
 // Per-tile frame lists of the object gather (host, from the positions).  The
 // tile height and the blocks per tile are chosen once, at the first build, so
-// that a small object does not leave most SMs idle.  A tile's frames are a
-// serial chain of copies: the tensor-copy gather (N >= 64) shares a tile among a
-// cluster of blocks when there are fewer than kFewTiles full tiles with at least
-// kLongChain copies each, and takes half tiles below half of that.
-// us per gather and normalisation:
-//                                 full tiles in clusters of | half tiles of
-//                                   1     2     4           |   1     2     4
-//   100 x  64^2 on  256^2 ( 64)    18    16    18           |  16    14    19
-//   150 x  64^2 on  162^2 ( 36)    52    32    23           |  46    29    19
-//   301 x 128^2 on  397^2 (169)    49    33    33           |  44    34    41
-//    97 x 192^2 on  420^2 (196)    37    27    30           |  35    29    37
-//    60 x 256^2 on  500^2 (250)    27    26    38           |  27    31    47
-//   500 x 256^2 on 1100^2          83   104   166           |  89   155   235
-// The plain gather halves the height while there are fewer tiles than two blocks
-// per SM.
-constexpr size_t kFewTiles = 250;
-constexpr size_t kLongChain = 12;
+// that a small object does not leave most SMs idle: half tiles below kFewTiles full
+// ones, and (tensor-copy gather, N >= 64) 1, 2 or 4 blocks to a tile, as a cluster.  A
+// tile's items (frames x modes) are a serial chain of copies, 0.33 us each, which
+// the blocks of a cluster share; all items together take 0.6 ns each; a cluster
+// costs 14 (two) or 38 ns (four) per tile.  gather_us adds the chain and the whole in
+// quadrature, which is within 10 % of the best choice over 80 scans of 64^2 to 256^2
+// with 20 to 3000 frames, and a larger cluster is taken where it saves a tenth by it.
+// Half tiles in clusters of 1 / 2 / 4, us:
+//    20 x  64^2 on  540^2   8.3  11.6  22.2  |    60 x 256^2 on 500^2  24.5  19.3  29.6
+//   100 x  64^2 on  256^2  14.4  12.2  15.6  |   200 x 256^2 on 500^2  67.7  43.4  43.3
+//   800 x  64^2 on  500^2  23.2  26.9  34.7  |   800 x 256^2 on 500^2   251   148   110
+//   150 x  64^2 on  162^2  44.4  26.7  18.4  |   301 x 128^2 on 397^2  42.5  28.3  26.7
+//  2441 x  64^2, K 2, 509  96.5  99.1  95.4  |  1562 x  80^2, K 2, 525 90.1  88.3  85.2
+// (these two on full tiles 131 and 107.)  The plain gather (N < 64) halves the height
+// while there are fewer tiles than two blocks per SM.
+constexpr size_t kFewTiles = 2 * 152;
+double gather_us(const TileLoad& t, int K, int blocks) {
+    const double chain = 0.33 * t.longest * K / blocks, all = 0.6e-3 * (double)t.pairs * K;
+    const double cluster = blocks == 1 ? 0.0 : (blocks == 2 ? 0.014 : 0.038) * (double)t.tiles;
+    return std::sqrt(chain * chain + all * all) + cluster;
+}
 void build_tiles(ProbHost& h, const int32_t* positions) {
     const ptx_problem& p = h.p;
     if (h.tile_h == 0) {
         h.tile_h = kObjTileH;
-        if (p.N >= 64) {
-            size_t pairs = 0;
-            const size_t n = active_tiles(p, positions, kObjTileW, kObjTileH, &pairs);
-            if (n < kFewTiles && pairs * p.K >= kLongChain * n) {
-                h.gather_split = 2;
-                if (n < kFewTiles / 2) {
-                    h.tile_h = kObjTileH / 2;
-                    if (active_tiles(p, positions, kObjTileW, h.tile_h) < 100) h.gather_split = 4;
-                }
-            } else if (n < kFewTiles) {
-                h.tile_h = kObjTileH / 2;
-            }
-        } else {
-            while (h.tile_h > kObjTileH / 4 && active_tiles(p, positions, kObjTileW, h.tile_h) < 2 * 152) h.tile_h /= 2;
+        const int least = p.N >= 64 ? kObjTileH / 2 : kObjTileH / 4;
+        TileLoad load = tile_load(p, positions, kObjTileW, h.tile_h);
+        // (tiles of fewer than three frames are done sooner whole: 20 x 128^2 on 600^2 8.3 us, half tiles 9.7)
+        const bool few = load.tiles < kFewTiles && (p.N < 64 || load.pairs >= 3 * load.tiles);
+        while (few && h.tile_h > least && load.tiles < kFewTiles) {
+            h.tile_h /= 2;
+            load = tile_load(p, positions, kObjTileW, h.tile_h);
         }
+        if (p.N >= 64 && few)
+            while (h.gather_split < 4 &&
+                   gather_us(load, p.K, 2 * h.gather_split) < 0.9 * gather_us(load, p.K, h.gather_split))
+                h.gather_split *= 2;
     }
     const int TW = kObjTileW, TH = h.tile_h;
     const int ntx = (p.Wo + TW - 1) / TW, nty = (p.Ho + TH - 1) / TH;

@@ -327,3 +327,28 @@ def test_large_frames_around_the_split_limit(N, J, lanes, batch):
         assert np.linalg.norm(a.cpu().numpy() - b) <= tol * np.linalg.norm(b)
     assert abs(llk[0] - rl) < 1e-6 * rl
     pb.close()
+
+
+# clusters of four blocks whose tiles have from one to all of the frames; two modes; one block per tile
+@pytest.mark.parametrize("N,K,J,far,side", [(64, 1, 120, 2, 300), (64, 2, 70, 1, 260), (128, 1, 150, 3, 400), (64, 1, 6, 2, 300)])
+def test_object_gather_of_uneven_tiles(N, K, J, far, side):
+    """Most frames on one spot and a few in the opposite corner, so that the blocks
+    that share a tile outnumber its frames there: object and probe of one AP
+    cycle against the oracle."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + J)
+    obj = (1 + 0.3 * crandn(rng, side, side)).astype(np.complex64)
+    probe = crandn(rng, K, N, N)
+    pos = rng.integers(0, 9, (J, 2)).astype(np.int32)
+    pos[:far] = side - N - np.arange(far)[:, None]
+    phi = oracle.obj_probe_to_psi(obj, probe, pos)
+    ic = (np.abs(np.fft.fft2(phi, norm="ortho")) ** 2).sum(1)
+    io = (ic * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+    o, p = dev(obj), dev(probe)
+    pb = Ptycho(o, p, dev(io), pos)
+    pb.ap(1)
+    ro, rp, _ = oracle.ap_cycle(obj, probe, oracle.Data.make(io, pos, None))
+    tol = 2.0 ** -24 * (8 * np.log2(N) + 12 + np.sqrt(J))  # as in test_whole_frame_cycles
+    for a, b in ((o, ro), (p, rp)):
+        assert np.linalg.norm(a.cpu().numpy() - b) < tol * np.linalg.norm(b)
+    pb.close()
