@@ -7,12 +7,10 @@
 // 100 frames leaves one block per SM, whose time is its chain of loads,
 // codelets and barriers.  N R threads hold one codelet each (8 pixels), every
 // transpose is in place (a column's second factor rewrites exactly the rows it
-// read) or within a warp, and a block loops over its frames with its pixels'
-// probe sums in registers, flushing them once.  Two blocks of 512 threads per
-// SM at 64^2 (some of the sums spill) beat one without spills: LLK of 6000 frames
-// 163 (three passes) -> 131 us (one block per SM: 163), DM cycle 609 -> 582 (625).
-// The cycles take it while every frame has a block of its own: 100 frames of 64^2,
-// five AP cycles, 180 -> 170 us.
+// read) or within a warp.  Two blocks of 512 threads per SM at 64^2.  The cycles take
+// it while every frame has a block of its own (100 frames of 64^2, five AP cycles,
+// 180 -> 170 us), whose probe terms go straight to the accumulators; the LLK's blocks
+// loop over more frames than that: 6000 frames 163 (three passes) -> 131 us.
 #pragma once
 #include "kernels_reg.cuh"
 
@@ -75,7 +73,7 @@ __device__ __noinline__ float frame_bright(const ProbArgs& a, int j) {
     return llk;
 }
 
-// grid (blocks): block x handles frames x, x + gridDim.x, ...
+// grid (blocks): block x handles frame x, FRAME_LLK also x + gridDim.x, ...
 template <int N, int kForm>
 __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r(const __grid_constant__ ProbArgs a, int upd_probe) {
     constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>(), T = frame_threads<N>();
@@ -98,13 +96,6 @@ __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r
         else
             __syncthreads();
     };
-    float2 np_r[M];
-    float dp_r[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        np_r[i] = make_float2(0.f, 0.f);
-        dp_r[i] = 0.f;
-    }
     uint32_t mbits = 0u;  // rows cn + R i of column c
 #pragma unroll
     for (int i = 0; i < M; ++i) mbits |= (a.mask[(cn + R * i) * N + c] != 0) ? (1u << i) : 0u;
@@ -201,28 +192,24 @@ __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r
                 const float2 prv = __ldg(a.probe + ls * N + x), obv = obj[(size_t)ls * a.Wo + x];
                 const float2 w = cadd(cmul(prv, obv), u[i]);
                 __stcs(psi + ls * N + x, w);
-                const float2 s = cconjmul(obv, w);
-                np_r[i].x += s.x;
-                np_r[i].y += s.y;
-                dp_r[i] += cnorm(obv);
+                if (upd_probe) {
+                    const float2 s = cconjmul(obv, w);
+                    red_add_v4(a.acc_probe + ls * N + x, s.x, s.y, cnorm(obv), 0.f);
+                }
             }
-            __syncthreads();  // the next frame's rows go into the same buffer
+            return;
         }
-    }
-    if (kForm != FRAME_LLK && upd_probe) {
-#pragma unroll
-        for (int i = 0; i < M; ++i) red_add_v4(a.acc_probe + ls * N + ks + R * i, np_r[i].x, np_r[i].y, dp_r[i], 0.f);
     }
 }
 
 template <int N>
 size_t smem_frame_r() { return sizeof(float2) * (N + (size_t)N * reg_pitch<N>()); }
 
-// form: FrameForm; all frames of the problem
+// form: FrameForm; all frames of the problem (but for FRAME_LLK no more than frame_blocks(N))
 template <int N>
 void launch_frame(const ProbArgs& a, int form, int upd_probe, cudaStream_t s) {
     if constexpr (frame_whole<N>()) {
-        const int grid = a.J < frame_blocks(N) ? a.J : frame_blocks(N);
+        const int grid = form != FRAME_LLK || a.J < frame_blocks(N) ? a.J : frame_blocks(N);
         auto k = form == FRAME_DM ? k_frame_r<N, FRAME_DM> : (form == FRAME_LLK ? k_frame_r<N, FRAME_LLK> : k_frame_r<N, FRAME_PHI>);
         k<<<grid, frame_threads<N>(), smem_frame_r<N>(), s>>>(a, upd_probe);
     }
