@@ -56,6 +56,24 @@ struct RegShape {
     static_assert(N % L == 0, "lines per block must divide N");
 };
 
+// Sizes whose LLK, cycles and gradient take the passes with the column transform
+// split between them (kernels_split.cuh).  At 128^2 half the threads of a split row
+// block idle in the 16-point factors (2500-frame LLK 228 -> 265 us).
+template <int N>
+__host__ __device__ constexpr bool use_split() {
+    return N >= 160;
+}
+// Whether the passes of this file have forms of their own there for several modes'
+// and a background's cycles and the object's gradient: only where something still
+// reaches them (above 256^2 the cycles of few frames of one mode); elsewhere the
+// general forms serve.
+template <int N>
+constexpr bool own_modes_cycle() { return !use_split<N>(); }
+template <int N>
+constexpr bool own_bg_cycle() { return !use_split<N>() || Plan<N>::M > Plan<N>::R; }
+template <int N>
+constexpr int own_grad() { return use_split<N>() ? 0 : 2; }
+
 // Row passes whose lines each stay within one warp (both factors fill the
 // warp's lanes with whole lines): the transpose between the two factors then
 // needs no block barrier, so that a block's warps drift apart and the loads of
@@ -735,32 +753,25 @@ cudaError_t set_attrs_ls() {
 }
 template <int N>
 cudaError_t set_attrs_r() {
-    cudaError_t e;
-    const int mx = 200 * 1024;
-    const int carve = cudaSharedmemCarveoutMaxShared;  // room for 5-6 blocks of ~37 KB per SM
-    if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_modes_r<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_modes_r<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_modes_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_modes_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_fwd_r<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_col_r<N, true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 0>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 1>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    if ((e = cudaFuncSetAttribute(k_row_bwd_r<N, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
-    return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto k) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        // room for 5-6 blocks of ~37 KB per SM
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    };
+    set(k_row_fwd_r<N, false>);
+    set(k_row_fwd_r<N, true>);
+    set(k_col_r<N, false, true>);
+    set(k_col_r<N, false, false>);
+    set(k_col_r<N, true, own_bg_cycle<N>()>);
+    set(k_col_r<N, true, false>);
+    set(k_col_modes_r<N, own_modes_cycle<N>()>);
+    set(k_col_modes_r<N, false>);
+    set(k_row_bwd_r<N, 0>);
+    set(k_row_bwd_r<N, 1>);
+    set(k_row_bwd_r<N, own_grad<N>()>);
+    return e;
 }
 
 }  // namespace ptx

@@ -27,23 +27,12 @@
 
 namespace ptx {
 
-// Sizes whose LLK, cycles and gradient take the split passes.  At 128^2 half the
-// threads of a row block idle in the 16-point factors (2500-frame LLK 228 -> 265 us);
-// its line search gains all the same (CG step of 900 frames 424 -> 389 us).
-template <int N>
-__host__ __device__ constexpr bool use_split() {
-    return N >= 160;
-}
+// Sizes whose line search takes them: 128^2 gains there (CG step of 900 frames 424 ->
+// 389 us), though not in its other passes (use_split, kernels_reg.cuh).
 template <int N>
 __host__ __device__ constexpr bool use_split_ls() {
     return N >= 128;
 }
-// sizes whose near-field passes are split too (the row pass at the detector keeps rows in a warp)
-template <int N>
-__host__ __device__ constexpr bool use_split_nf() {
-    return N == 256;
-}
-
 template <int N>
 struct SplitShape {
     static constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>();
@@ -57,6 +46,11 @@ struct SplitShape {
     static constexpr int RowBlocks = M > 16 ? 2 : 5;
     static constexpr int ColBlocks = M > 16 ? 2 : 4;
 };
+// sizes whose near-field passes are split too: k_row_proj_s keeps its rows in a warp
+template <int N>
+__host__ __device__ constexpr bool use_split_nf() {
+    return use_split<N>() && SplitShape<N>::kWarpRows;
+}
 template <int N>
 __device__ __forceinline__ void split_row_sync() {
     if constexpr (SplitShape<N>::kWarpRows)
