@@ -645,16 +645,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_row_bwd_s(ProbArgs a, int j0, i
     }
 }
 
-// Sixteen 32-bit words per thread of a warp in tensor memory, and the waits for
-// them (the warp's lanes of its quarter, columns from addr on).
+// Sixteen 32-bit words per thread of a warp in tensor memory (the warp's lanes of its
+// quarter, columns from addr on).  A load and its wait are one statement, so that
+// nothing that uses the values can be moved in between.
 __device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
     uint32_t r[16];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(addr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        : "r"(addr)
+        : "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
