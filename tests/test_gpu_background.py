@@ -139,3 +139,43 @@ def test_background_under_an_infinite_model_intensity(N, K, nf):
     io = np.full((N, N), 7.0, np.float32)
     got = _background_only(io, np.full((N, N), 5.0, np.float32), probe)
     assert np.all(got == 0.0)
+
+
+# remainders of M by four (160, 224, 400), several modes, the near field with and without split passes, few large
+# frames (unsplit) and more (split); odd frame counts in one batch, and in batches of 5 (dependent launches)
+@pytest.mark.parametrize("N,K,J,nf", [(64, 2, 9, 0.0), (80, 1, 21, 0.0), (128, 2, 7, 0.0), (160, 1, 23, 0.0), (160, 2, 11, 0.0),
+                                      (224, 1, 11, 0.0), (256, 1, 13, 0.0), (256, 2, 7, 0.0), (400, 1, 7, 0.0),
+                                      (400, 1, 11, 0.0), (400, 2, 5, 0.0), (512, 1, 9, 0.0), (512, 2, 3, 0.0),
+                                      (128, 1, 9, 40.0), (256, 1, 13, 90.0)])
+@pytest.mark.parametrize("batch", [0, 5])
+def test_background_update_in_every_pass(N, K, J, nf, batch):
+    """One AP cycle that updates object, probe and background, with a mask,
+    against the oracle."""
+    from paper_2008_11511_gb300 import Ptycho
+    rng = np.random.default_rng(N + 10 * K + J)
+
+    def crandn(*shape):
+        return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+    Ho, Wo = N + 21, N + 18
+    obj, probe = (1 + 0.3 * crandn(Ho, Wo)).astype(np.complex64), crandn(K, N, N)
+    pos = np.stack([rng.integers(0, Ho - N + 1, J), rng.integers(0, Wo - N + 1, J)], 1).astype(np.int32)
+    mask = (rng.random((N, N)) < 0.1).astype(np.uint8)
+    empty = oracle.Data.make(np.zeros((J, N, N), np.float32), pos, mask, nearfield=nf)
+    ic = (np.abs(empty.to_detector(oracle.obj_probe_to_psi(obj, probe, pos))) ** 2).sum(1)
+    bg = (ic.mean() * rng.uniform(0.5, 1.5, (N, N))).astype(np.float32)
+    io = ((ic + bg) * rng.uniform(0.3, 2.0, ic.shape)).astype(np.float32)
+    io[:, mask.astype(bool)] = 0.0
+    pb = Ptycho(dev(obj), dev(probe), dev(io), pos, mask, background=dev(bg), nearfield=nf)
+    pb.set_param("batch_frames", batch)
+    llk = pb.ap(1, update_background=True).cpu().numpy()
+    ro, rp, rb, rl = oracle.ap_cycle_background(obj, probe, bg, oracle.Data.make(io, pos, mask, nearfield=nf))
+    # single precision: 4 transforms (near field 8) of log2 N levels and a dozen roundings, each 2^-24 of the rms;
+    # the sums add J terms in FP32.  The background is the mean of J quotients of wave intensities, twice the waves'
+    # relative errors
+    tol = 2.0 ** -24 * ((16 if nf else 8) * np.log2(N) + 12 + np.sqrt(J))
+    assert rel(pb.obj.cpu().numpy(), ro) < tol and rel(pb.probe.cpu().numpy(), rp) < tol
+    assert rel(pb.background.cpu().numpy(), rb) < 2 * tol
+    assert abs(llk[0] - rl) < 1e-6 * abs(rl)
+    assert np.array_equal(pb.background.cpu().numpy()[mask.astype(bool)], bg[mask.astype(bool)])
+    pb.close()
