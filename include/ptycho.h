@@ -301,8 +301,10 @@ ptx_status ptx_position_shifts(ptx_handle* h, int32_t p, float filter_ratio, flo
 ptx_status ptx_set_positions(ptx_handle* h, int32_t p, const int32_t* positions, void* stream);
 
 /* Per-kernel timing for measurement.  While enabled, the cycle calls launch
- * their kernels directly (no CUDA graph) and bracket every launch with CUDA
- * events recorded on the launch stream.  Enabling resets the counters. */
+ * their kernels directly (no CUDA graph) in one lane and bracket every launch
+ * with CUDA events recorded on the launch stream; frames of 32 and 64, whose
+ * cycle is one launch over whole frames otherwise, take the three passes.
+ * Enabling resets the counters. */
 ptx_status ptx_profile_enable(ptx_handle* h, int32_t enable);
 
 /* Wait for the recorded events and return, for each of the first `nkinds`

@@ -334,9 +334,9 @@ ptx_status check_problem(const ptx_problem& p, int idx) {
 // line search in 62 -> 56 frames, 3.68 -> 3.61 ms.  Several lanes fill each other's
 // tails (4000 x 256^2 DM cycle: 48 to 64 frames are within 1 %, whole waves of 38
 // frames 2 % slower), so there it is `most` frames, then the rest, unless a few
-// batches of few frames would leave a lane idle at the end (with many frames to a
-// batch little is lost, and evening them would regroup the probe's sums): 30 x 400^2 in 13 + 13 + 4 frames 376 us,
-// in 4 x 8 333; 107 x 512^2 in 6 x 16 + 11 497, in 8 x 14 468.
+// batches of few frames would leave a lane idle at the end: 30 x 400^2 in 13 + 13 + 4
+// frames 376 us, in 4 x 8 333; 107 x 512^2 in 6 x 16 + 11 497, in 8 x 14 468.  (With many
+// frames to a batch little is lost, and evening them would regroup the probe's sums.)
 constexpr size_t kFewFrames = 32;
 size_t even_batch(size_t most, size_t J, int lanes, double wave) {
     most = std::max<size_t>(1, std::min<size_t>(most, 32768));  // grid.y limit of the batch kernels
@@ -1461,8 +1461,8 @@ ptx_status ptx_ml_grad(ptx_handle* h, void* grad_obj, void* grad_probe, double* 
         (split ? ph.ks->row_fwd_s : ph.ks->row_fwd)(a, j0, nb, X_PHI, s, pdl && j0 > 0);
         (split ? ph.ks->col_s : ph.ks->col)(a, j0, nb, COL_GRAD, s, pdl);
         if (grad_obj || grad_probe)
-            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, grad_obj != nullptr, grad_probe != nullptr, s,
-                           pdl);
+            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, grad_obj != nullptr,
+                                                        grad_probe != nullptr, s, pdl);
     }
     if (llk_dev) k_llk_sum<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, a, a.N / a.C2, llk_dev);
     e = cudaGetLastError();
@@ -1541,7 +1541,8 @@ ptx_status enqueue_grad(ptx_handle* h, ProbHost& ph, float2* g_obj, float2* g_pr
         (split ? ph.ks->row_fwd_s : ph.ks->row_fwd)(a, j0, nb, X_PHI, s, pdl && j0 > 0);
         (split ? ph.ks->col_s : ph.ks->col)(a, j0, nb, COL_GRAD, s, pdl);
         if (g_obj || g_probe)
-            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, g_obj != nullptr, g_probe != nullptr, s, pdl);
+            (split ? ph.ks->row_bwd_s : ph.ks->row_bwd)(a, j0, nb, std::min(ph.G3, nb), BWD_GRAD, g_obj != nullptr,
+                                                        g_probe != nullptr, s, pdl);
     }
     if (llk_out) k_llk_sum<<<kCycleEndBlocks, 256, 0, s>>>(h->ctl, a, a.N / a.C2, llk_out);
     e = cudaGetLastError();

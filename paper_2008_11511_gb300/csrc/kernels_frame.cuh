@@ -75,7 +75,8 @@ __device__ __noinline__ float frame_bright(const ProbArgs& a, int j) {
 
 // grid (blocks): block x handles frame x, FRAME_LLK also x + gridDim.x, ...
 template <int N, int kForm>
-__global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r(const __grid_constant__ ProbArgs a, int upd_probe) {
+__global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4)
+    k_frame_r(const __grid_constant__ ProbArgs a, int upd_probe) {
     constexpr int R = Plan<N>::R, M = Plan<N>::M, P = reg_pitch<N>(), T = frame_threads<N>();
     constexpr bool kWarp = R == M && 32 % R == 0;  // a row's threads are in one warp in both factors
     extern __shared__ __align__(16) float2 sm[];
@@ -84,8 +85,8 @@ __global__ void __launch_bounds__(frame_threads<N>(), N >= 64 ? 2 : 4) k_frame_r
     float2* buf = sm + N;
     load_twiddles<N>(tw);
     const int t = threadIdx.x;
-    // the thread's items: first factor of a row (lf, nf) and of a column (column cf,
-    // rows n + M i), second factor of a row (ls, ks) and of a column (cs, ...)
+    // the thread's items: first factor of a row (lf, nf), second factor of a row (ls, ks),
+    // either factor of a column (c, cn)
     const bool f = t < N * M;                    // first-factor items (all threads when R == M)
     const int lf = t / M, nf = t - lf * M;       // row lf, elements nf + M i
     const int ls = t / R, ks = t - ls * R;       // row ls, elements ks + R i
@@ -210,7 +211,9 @@ template <int N>
 void launch_frame(const ProbArgs& a, int form, int upd_probe, cudaStream_t s) {
     if constexpr (frame_whole<N>()) {
         const int grid = form != FRAME_LLK || a.J < frame_blocks(N) ? a.J : frame_blocks(N);
-        auto k = form == FRAME_DM ? k_frame_r<N, FRAME_DM> : (form == FRAME_LLK ? k_frame_r<N, FRAME_LLK> : k_frame_r<N, FRAME_PHI>);
+        auto k = form == FRAME_DM    ? k_frame_r<N, FRAME_DM>
+                 : form == FRAME_LLK ? k_frame_r<N, FRAME_LLK>
+                                     : k_frame_r<N, FRAME_PHI>;
         k<<<grid, frame_threads<N>(), smem_frame_r<N>(), s>>>(a, upd_probe);
     }
 }

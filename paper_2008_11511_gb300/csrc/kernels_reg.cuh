@@ -220,7 +220,8 @@ __device__ __noinline__ float col_bright_r(const ProbArgs& a, int j0, int bx, in
 // cycle's projection (COL_PROJECT) fixed at compile time; otherwise the mode
 // comes from the argument.
 template <int N, bool kBg, bool kCycle>
-__global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks) k_col_r(const __grid_constant__ ProbArgs a, int j0, int mode_arg) {
+__global__ void __launch_bounds__(kThreads, RegShape<N>::ColMinBlocks)
+    k_col_r(const __grid_constant__ ProbArgs a, int j0, int mode_arg) {
 #define PTX_BX blockIdx.x
 #define PTX_BY blockIdx.y
 #define PTX_GX gridDim.x

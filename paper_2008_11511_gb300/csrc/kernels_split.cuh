@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(SplitShape<N>::TC, SplitShape<N>::ColBlocks * 
 #pragma unroll
     for (int n1 = 0; n1 < M; ++n1) u[n1] = ld_hint(spec + n1 * RN, el);
     Dft<M, -1>::run(u);
-    float llk = project_pixels<N, kBg, false>(u, io, mbits, mode, kBg ? a.bg + id : nullptr, a.bg_acc + id, a.bg_acc != nullptr);
+    float llk = project_pixels<N, kBg, false>(u, io, mbits, mode, kBg ? a.bg + id : nullptr, a.bg_acc + id,
+                                              a.bg_acc != nullptr);
     if (__all_sync(0xffffffffu, llk < kInf)) {
         if (mode != COL_LLK) {
             Dft<M, +1>::run(u);
@@ -413,7 +414,8 @@ __global__ void __launch_bounds__(kThreads, SplitShape<N>::RowBlocks) k_row_fwd_
 // Line search, column pass (k_col_ls_r's sums): second factors of every wave of
 // the thread's pixels.  grid (N / C, frames in batch)
 template <int N, bool kModes, bool kThree>
-__global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, kThree>() * kThreads + SplitShape<N>::TC - 1) / SplitShape<N>::TC)
+__global__ void __launch_bounds__(SplitShape<N>::TC, (ls_min_blocks<N, kModes, kThree>() * kThreads + SplitShape<N>::TC - 1) /
+                                                         SplitShape<N>::TC)
     k_col_ls_s(ProbArgs a, int j0) {
     using S = SplitShape<N>;
     constexpr int R = S::R, M = S::M, RN = R * N, kWaves = kThree ? 3 : 2;
@@ -910,7 +912,8 @@ void launch_row_bwd_s(const ProbArgs& a, int j0, int nb, int G, int mode, int up
 // Near field (pdl: as for the passes above) and line search.
 template <int N>
 void launch_col_nf_s(const ProbArgs& a, int nb, int dir, cudaStream_t s, bool pdl) {
-    launch_dep<SplitShape<N>::TC>(dir < 0 ? k_col_nf_s<N, -1> : k_col_nf_s<N, +1>, dim3(N / reg_cols<N>(), nb), 0, s, pdl, a);
+    launch_dep<SplitShape<N>::TC>(dir < 0 ? k_col_nf_s<N, -1> : k_col_nf_s<N, +1>, dim3(N / reg_cols<N>(), nb), 0, s, pdl,
+                                  a);
 }
 template <int N>
 void launch_row_proj_s(const ProbArgs& a, int j0, int nb, int llk_only, cudaStream_t s, bool pdl) {
