@@ -352,3 +352,21 @@ def test_object_gather_of_uneven_tiles(N, K, J, far, side):
     for a, b in ((o, ro), (p, rp)):
         assert np.linalg.norm(a.cpu().numpy() - b) < tol * np.linalg.norm(b)
     pb.close()
+
+
+@pytest.mark.parametrize("N,K", [(256, 1), (512, 1), (512, 2)])
+@pytest.mark.parametrize("form", [1, 2])
+def test_tensor_core_projection_of_a_faint_wave(N, K, form):
+    """test_projection_of_a_faint_wave_on_bright_pixels in the tensor-core forms."""
+    from paper_2008_11511_gb300 import Ptycho
+    probe = np.zeros((K, N, N), np.complex64)
+    probe[K - 1, 0, 0] = N * np.sqrt(1e-29)
+    io = np.full((1, N, N), 1e11, np.float32)
+    pb = Ptycho(dev(np.ones((N, N), np.complex64)), dev(probe), dev(io), np.zeros((1, 2), np.int32), None)
+    pb.set_param("tc", form)
+    llk = float(pb.ap(1, update_obj=False, update_probe=False)[0])
+    want = N * np.sqrt(1e11)
+    assert abs(pb.psi.cpu().numpy()[0, K - 1, 0, 0] - want) < 1e-5 * want  # the forms' tolerance in the parity tests
+    ref = N * N * oracle.llk_terms(np.array([1e-29]), np.array([1e11]), np.zeros(1, bool))[0]
+    assert abs(llk - ref) < 1e-5 * ref
+    pb.close()
