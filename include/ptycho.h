@@ -274,7 +274,7 @@ ptx_status ptx_fft2(void* data, int32_t nframes, int32_t N, int32_t direction, v
 #define PTX_KERNEL_ROW_FWD   0 /* gather x probe, (2 Phi - Psi), forward row FFT */
 #define PTX_KERNEL_COL       1 /* column FFT, amplitude projection + LLK, inverse column FFT */
 #define PTX_KERNEL_ROW_BWD   2 /* inverse row FFT, Psi update, probe numerator / denominator */
-#define PTX_KERNEL_DEN_MAX   3 /* max of the denominators */
+#define PTX_KERNEL_DEN_MAX   3 /* max of the denominators (part of PTX_KERNEL_NORMALISE for probes up to 16384 pixels) */
 #define PTX_KERNEL_NORMALISE 4 /* normalisation of O and P */
 #define PTX_KERNEL_CYCLE_END 5 /* FP64 LLK reduction of the cycle */
 #define PTX_KERNEL_OBJ_GATHER 6 /* object numerator / denominator gathered per tile from Psi' */

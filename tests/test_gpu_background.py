@@ -179,3 +179,17 @@ def test_background_update_in_every_pass(N, K, J, nf, batch):
     assert abs(llk[0] - rl) < 1e-6 * abs(rl)
     assert np.array_equal(pb.background.cpu().numpy()[mask.astype(bool)], bg[mask.astype(bool)])
     pb.close()
+
+
+@pytest.mark.parametrize("N,K,nf", FORMS + [(128, 1, 30.0), (256, 1, 90.0)])
+def test_background_is_added_once_beside_bright_pixels(N, K, nf):
+    """Some pixels so bright over their model (1e9 counts, 1e-29) that their
+    neighbours' likelihood is computed again: the background's sums are not."""
+    rng = np.random.default_rng(N + K)
+    bg = rng.uniform(1.0, 100.0, (N, N)).astype(np.float32)
+    io = rng.uniform(1.0, 100.0, (N, N)).astype(np.float32)
+    y, x = rng.integers(0, N, (2, 9))
+    bg[y, x], io[y, x] = 1e-29, 1e9
+    got = _background_only(io, bg, np.zeros((K, N, N), np.complex64), nf)
+    # a unit in the last place of the quotient and the rounding of the product
+    assert np.abs(got.astype(np.float64) / io - 1).max() <= 2.0 ** -22

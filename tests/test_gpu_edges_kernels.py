@@ -370,3 +370,21 @@ def test_tensor_core_projection_of_a_faint_wave(N, K, form):
     ref = N * N * oracle.llk_terms(np.array([1e-29]), np.array([1e11]), np.zeros(1, bool))[0]
     assert abs(llk - ref) < 1e-5 * ref
     pb.close()
+
+
+@pytest.mark.parametrize("N", [128, 256])
+@pytest.mark.parametrize("param", ["persistent", "tma"])
+def test_faint_wave_in_the_other_schedules(N, param):
+    """The same in the persistent schedule and the column pass fed by tensor copies."""
+    from paper_2008_11511_gb300 import Ptycho
+    probe = np.zeros((1, N, N), np.complex64)
+    probe[0, 0, 0] = N * np.sqrt(1e-29)
+    io = np.full((2, N, N), 1e11, np.float32)
+    pb = Ptycho(dev(np.ones((N, N), np.complex64)), dev(probe), dev(io), np.zeros((2, 2), np.int32), None)
+    pb.set_param(param, 1)
+    llk = float(pb.ap(1, update_obj=False, update_probe=False)[0])
+    want = N * np.sqrt(1e11)
+    assert np.abs(pb.psi.cpu().numpy()[:, 0, 0, 0] - want).max() < 2.0 ** -20 * want
+    ref = 2 * N * N * oracle.llk_terms(np.array([1e-29]), np.array([1e11]), np.zeros(1, bool))[0]
+    assert abs(llk - ref) < 2.0 ** -20 * ref
+    pb.close()
